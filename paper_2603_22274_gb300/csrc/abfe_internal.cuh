@@ -51,6 +51,10 @@ constexpr double FSCALE = 4294967296.0;
 constexpr float FSCALEF = 4294967296.0f;
 constexpr double INV_FSCALE = 1.0 / 4294967296.0;
 constexpr float DUMMY_FAR = 1.0e4f;
+// j-cluster entries per ligand work item (a warp each). Shorter than the
+// environment's: one window's ligand has some 2,300 entries in all, and in items
+// of 16 they kept 144 of the chip's 608 schedulers busy for 25 us.
+constexpr int LIG_CHUNK = 8;
 
 // error bits (Counters::err)
 enum : int {
@@ -140,7 +144,7 @@ struct RepDev {
 
 struct BoreschDev {
     int anc[6];
-    double r0, th0[2], ph0[3], kr, kth, kph;
+    double r0, th0[2], cph0[3], sph0[3], kr, kth, kph;   // cos and sin of the phi0
 };
 
 struct Item {
@@ -239,7 +243,7 @@ struct DevPtrs {
     int n_bond_total;              // bonds of all replicas
     const BoreschDev* bor;
     const int4* sys_tors;          // torsion atoms a, b, c, d (original indices)
-    const dbl4* sys_torsp;         // k, n, phi0, -
+    const dbl4* sys_torsp;         // k, n, cos phi0, sin phi0
     const int* sys_aw;             // alchemical oxygens (original indices), per system
     const float* sys_dq;           // per system atom: dq sqrt(k_e) (0 unless an alchemical oxygen)
     const double* sys_dqd;         // the same in e, FP64
@@ -423,7 +427,7 @@ void launch_rebuild(const DevPtrs& P, cudaStream_t s, int n_sm);
 void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl);
 void launch_prune(const DevPtrs& P, cudaStream_t s, int n_sm);
 void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precision, int grid,
-                       int block);
+                       int block, int n_sm);
 int env_kernel_occupancy(int block, int precision, bool energy);
 void launch_lig_forces(const DevPtrs& P, cudaStream_t s, int precision, int grid, int block,
                        bool energy);
@@ -435,11 +439,10 @@ void launch_step_end(const DevPtrs& P, cudaStream_t s, int inc_step, int force_r
                      cudaGraphConditionalHandle h_prune, cudaGraphConditionalHandle h_exchange,
                      int use_handle);
 void launch_bonds(const DevPtrs& P, cudaStream_t s, int precision, bool energy);
-void launch_torsions(const DevPtrs& P, cudaStream_t s, int max_tors);
 // alchemical waters: slot charges at every replica's lambda_q; energy-pass sums
 void launch_aw_refresh(const DevPtrs& P, cudaStream_t s);
 void launch_aw_sums(const DevPtrs& P, cudaStream_t s, int max_aw);
-void launch_boresch(const DevPtrs& P, cudaStream_t s);
+void launch_restraints(const DevPtrs& P, cudaStream_t s);
 void launch_finalize(const DevPtrs& P, cudaStream_t s);
 void launch_ukn_assemble(const DevPtrs& P, cudaStream_t s, double kT);
 void launch_scatter_out(const DevPtrs& P, cudaStream_t s, int what, double* outd, float* outf,

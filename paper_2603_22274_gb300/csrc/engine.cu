@@ -54,8 +54,9 @@ struct abfe_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaStream_t side = nullptr;
-    cudaStream_t fork = nullptr;           // ligand / bonded / restraint branch
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaStream_t fork = nullptr;           // ligand pair / bond branch
+    cudaStream_t fork2 = nullptr;          // restraint / torsion / PME branch
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     int device = 0, n_sm = 0;
     abfe_params prm{};
     abfe_tuning tune{};
@@ -69,8 +70,9 @@ struct abfe_ctx {
     std::vector<int> rep_of_cl_h;
     std::vector<int64_t> rep_atom_off;
     int64_t total_atoms = 0;
-    int S = 0, C = 0, NCOL = 0, max_bonds = 0, n_lig_cl = 0, max_lig_cl = 0, max_tors = 0;
+    int S = 0, C = 0, NCOL = 0, max_bonds = 0, n_lig_cl = 0, max_lig_cl = 0;
     int n_bond_total = 0;
+    int64_t epc_max = 0;                   // outer entries per cluster, the largest estimate
     int max_aw = 0;
     std::vector<int> sys_tors_off, sys_ntors, sys_aw_off, sys_naw;
     DevPtrs P{};
@@ -306,33 +308,43 @@ DevPtrs with_sp(const abfe_ctx* c, int slot) {
     return P;
 }
 
-// The small ligand, bond and restraint kernels run on a forked stream next to
-// the environment pair kernel (parallel branches when captured in a graph);
-// all of them add into the same fixed-point force accumulators.
-// (fork = false: everything on s, for captures where the fork stream is busy)
+// The other force kernels run on forked streams next to the environment pair
+// kernel (parallel branches when captured in a graph): ligand pairs and bonds
+// on one; the FP64 bonded terms and the alchemical-water sums, or PME, on the
+// other (each is a chain of latency-bound launches: one after the other on a single
+// fork they were longer than the environment kernel of a 60,000-atom window,
+// 107 against 72 us). All of them add into the same fixed-point force
+// accumulators. (fork = false: everything on s, for captures where the fork
+// streams are busy)
 void enqueue_forces(abfe_ctx* c, cudaStream_t s, bool energy, bool fork = true) {
-    cudaStream_t f = fork ? c->fork : s;
+    cudaStream_t f = fork ? c->fork : s, f2 = fork ? c->fork2 : s;
     if (fork) {
         cudaEventRecord(c->ev_fork, s);
         cudaStreamWaitEvent(c->fork, c->ev_fork, 0);
+        cudaStreamWaitEvent(c->fork2, c->ev_fork, 0);
     }
     if (fork) prof_rec(c, c->ev_lig, true, f);
     launch_lig_forces(c->P, f, c->prm.precision, c->lig_grid, 128, energy);
     if (fork) prof_rec(c, c->ev_lig, false, f);
     launch_bonds(c->P, f, c->prm.precision, energy);
-    launch_torsions(c->P, f, c->max_tors);
-    launch_boresch(c->P, f);
-    if (energy) launch_aw_sums(c->P, f, c->max_aw);
+    launch_restraints(c->P, c->pme ? f : f2);
+    if (energy) launch_aw_sums(c->P, f2, c->max_aw);
     if (c->pme) {
-        launch_pme_forces(c->P, c->pm, f, c->n_sm, energy);
+        launch_pme_forces(c->P, c->pm, f2, c->n_sm, energy);
         // energy passes also split the reciprocal energy by charge kind (dU/dlambda_q, u_kn)
-        if (energy) launch_pme_decomposition(c->P, c->pm, f, c->n_sm);
+        if (energy) launch_pme_decomposition(c->P, c->pm, f2, c->n_sm);
     }
-    if (fork) cudaEventRecord(c->ev_join, c->fork);
+    if (fork) {
+        cudaEventRecord(c->ev_join, c->fork);
+        cudaEventRecord(c->ev_join2, c->fork2);
+    }
     if (fork) prof_rec(c, c->ev_env, true, s);
-    launch_env_forces(c->P, s, energy, c->prm.precision, c->env_grid, c->tune.block_threads);
+    launch_env_forces(c->P, s, energy, c->prm.precision, c->env_grid, c->tune.block_threads, c->n_sm);
     if (fork) prof_rec(c, c->ev_env, false, s);
-    if (fork) cudaStreamWaitEvent(s, c->ev_join, 0);
+    if (fork) {
+        cudaStreamWaitEvent(s, c->ev_join, 0);
+        cudaStreamWaitEvent(s, c->ev_join2, 0);
+    }
 }
 
 // zero forces, displacement check, rebuild and prune decisions, (predicated)
@@ -596,8 +608,16 @@ void update_grids(abfe_ctx* c) {
     c->P.skin_in_half2 = (float)(0.25 * c->tune.prune_skin * c->tune.prune_skin);
     int occ = env_kernel_occupancy(c->tune.block_threads, c->prm.precision, false);
     if (occ < 1) occ = 1;
-    c->env_grid = c->n_sm * occ;
-    c->lig_grid = c->n_sm * 4;
+    // as many blocks as the items can use (estimates from the outer list's size; the
+    // kernels claim what is left over): blocks without work still took registers
+    // from the kernels beside them (one solvent window: 53 us of pair kernel next to
+    // its forked neighbours, 37 alone)
+    const int warps = c->tune.block_threads / 32;
+    const int64_t items = (int64_t)c->C * (1 + c->epc_max / c->tune.max_entries);
+    c->env_grid = (int)std::min<int64_t>((int64_t)c->n_sm * occ,
+                                         std::max<int64_t>(c->n_sm, (items + warps - 1) / warps));
+    const int64_t lig_items = (int64_t)c->n_lig_cl * (1 + 2 * c->epc_max / LIG_CHUNK);
+    c->lig_grid = (int)std::min<int64_t>(c->n_sm * 4, std::max<int64_t>(1, (lig_items + 3) / 4));
     c->P.group = c->prm.precision == 1 ? 1 : c->tune.group;
     c->P.max_entries = c->tune.max_entries;
 }
@@ -810,8 +830,10 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
     }
     cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
     cudaStreamCreateWithFlags(&c->fork, cudaStreamNonBlocking);
+    cudaStreamCreateWithFlags(&c->fork2, cudaStreamNonBlocking);
     cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
+    cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming);
     c->tune.group = p->precision == 1 ? 1 : 2;
     c->tune.max_entries = 64;
     c->tune.block_threads = 128;
@@ -885,18 +907,21 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         }
         c->sys_tors_off.push_back((int)h_tors.size());
         c->sys_ntors.push_back(d.n_torsions);
-        c->max_tors = std::max(c->max_tors, d.n_torsions);
         for (int k = 0; k < d.n_torsions; ++k) {
             const int32_t* q = d.torsion_idx + 4 * k;
             h_tors.push_back(make_int4(q[0], q[1], q[2], q[3]));
-            h_torsp.push_back(dbl4{d.torsion_k[k], (double)d.torsion_n[k], d.torsion_phi0[k], 0.0});
+            h_torsp.push_back(dbl4{d.torsion_k[k], (double)d.torsion_n[k], std::cos(d.torsion_phi0[k]),
+                                   std::sin(d.torsion_phi0[k])});
         }
         if (d.has_boresch) {
             BoreschDev B;
             for (int a = 0; a < 6; ++a) B.anc[a] = d.anchors[a];
             B.r0 = d.b_r0;
             B.th0[0] = d.b_theta0[0]; B.th0[1] = d.b_theta0[1];
-            B.ph0[0] = d.b_phi0[0]; B.ph0[1] = d.b_phi0[1]; B.ph0[2] = d.b_phi0[2];
+            for (int a = 0; a < 3; ++a) {
+                B.cph0[a] = std::cos(d.b_phi0[a]);
+                B.sph0[a] = std::sin(d.b_phi0[a]);
+            }
             B.kr = d.b_kr; B.kth = d.b_ktheta; B.kph = d.b_kphi;
             c->sys_bor.push_back((int)h_bor.size());
             h_bor.push_back(B);
@@ -955,6 +980,7 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         c->sys_of_rep.push_back(s);
         for (int k = 0; k < R.n_cl_cap; ++k) c->rep_of_cl_h.push_back(r);
         const int64_t epc = est_entries_per_cluster(rho, rlist_cap, R.n_cl_cap);
+        c->epc_max = std::max(c->epc_max, epc);
         cap_e += (int64_t)R.n_cl_cap * epc;
         cap_x += 2LL * c->sys_nexcl[s] + 2LL * R.n_cl_cap + 64;
         h_ent_cap.push_back(std::max<int64_t>((int64_t)R.n_cl_cap * epc, 64));
@@ -973,10 +999,10 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         // bounding box is as long as its stretch of the chain, so no density
         // estimate bounds it: size the ligand items for every cluster of the
         // replica under every periodic image that can reach (3 per axis whose
-        // box edge is below 2 r_list + 3 nm), in items of at most 16 entries.
+        // box edge is below 2 r_list + 3 nm), in items of at most LIG_CHUNK entries.
         int64_t n_img = 1;
         for (int k = 0; k < 3; ++k) n_img *= d.box[k] < 2.0 * rlist_cap + 3.0 ? 3 : 1;
-        const int64_t lig_items = nlc ? (int64_t)nlc * (((int64_t)R.n_cl_cap * n_img + 15) / 16 + 1) + 4 : 4;
+        const int64_t lig_items = nlc ? (int64_t)nlc * (((int64_t)R.n_cl_cap * n_img + LIG_CHUNK - 1) / LIG_CHUNK + 1) + 4 : 4;
         cap_items_lig += lig_items;
         h_ilig_cap.push_back(lig_items);
         cl_off += R.n_cl_cap;
@@ -1355,8 +1381,10 @@ void abfe_destroy(abfe_ctx* c) {
     free_all(c);
     if (c->side) cudaStreamDestroy(c->side);
     if (c->fork) cudaStreamDestroy(c->fork);
+    if (c->fork2) cudaStreamDestroy(c->fork2);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
+    if (c->ev_join2) cudaEventDestroy(c->ev_join2);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
 }
@@ -2236,7 +2264,7 @@ abfe_status abfe_autotune(abfe_ctx* c, const char* cache_path, int32_t reps) {
             launch_prune(c->P, c->stream, c->n_sm);
             cudaEventRecord(e1, c->stream);
             launch_env_forces(c->P, c->stream, false, c->prm.precision, c->env_grid,
-                              t.block_threads);
+                              t.block_threads, c->n_sm);
             cudaEventRecord(e2, c->stream);
             cudaEventSynchronize(e2);
             c->force_prune = false;
@@ -2362,7 +2390,7 @@ abfe_status abfe_autotune_cadence(abfe_ctx* c, double dt, double gamma, uint64_t
         cudaEventElapsedTime(&b, e1, e2);
         cudaEventRecord(e0, c->stream);
         launch_env_forces(c->P, c->stream, false, c->prm.precision, c->env_grid,
-                          c->tune.block_threads);
+                          c->tune.block_threads, c->n_sm);
         cudaEventRecord(e1, c->stream);
         cudaEventSynchronize(e1);
         cudaEventElapsedTime(&e, e0, e1);

@@ -562,7 +562,7 @@ __device__ __noinline__ void lb_flush(const DevPtrs& P, LBS<ECAP, HCAP, XCAP, GM
         written += __popc(b);
     }
     if (n_plain + n_x == 0) return;
-    const int chunk = is_lig ? min(P.max_entries, 16) : P.max_entries;
+    const int chunk = is_lig ? LIG_CHUNK : P.max_entries;
     const int n_items = max(1, (n_plain + chunk - 1) / chunk);
     int ib = 0;
     if (lane == 0) ib = atomicAdd(is_lig ? &P.n_items_lig_r[r] : &P.n_items_env_r[r], n_items);

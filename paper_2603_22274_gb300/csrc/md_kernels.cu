@@ -8,11 +8,10 @@
 // * k_step_end: step counter, rebuild and prune flags, optional CUDA-graph
 //   conditionals.
 // * k_bonds: harmonic bonds (keep the synthetic molecules together).
-// * k_boresch: the six-term Boresch restraint in FP64, one thread per replica
-//   (paper, section "Restraints").
-// * k_torsions: periodic torsions of the ligand's rotatable bonds, scaled by
-//   lambda_v when annihilating (paper, section "Double annihilation protocol"),
-//   FP64, one thread per torsion.
+// * k_restraints: the FP64 bonded terms, a block per replica: the six-term Boresch
+//   restraint (paper, section "Restraints") and the periodic torsions of the
+//   ligand's rotatable bonds, scaled by lambda_v when annihilating (paper,
+//   section "Double annihilation protocol").
 // * k_aw_refresh / k_aw_sums: alchemical waters (paper, section "Double
 //   annihilation protocol"): their oxygens' slot charges at every replica's
 //   lambda_q, and on energy passes the pair sums that give their part of
@@ -409,7 +408,7 @@ __global__ void __launch_bounds__(256) k_bonds(DevPtrs P) {
     }
 }
 
-// ------------------------------------------------------------------ Boresch (FP64)
+// ------------------------------------------------------------------ restraint and torsions (FP64)
 struct D3 {
     double x, y, z;
 };
@@ -421,150 +420,166 @@ __device__ __forceinline__ D3 d3cross(D3 a, D3 b) {
 __device__ __forceinline__ D3 d3scale(D3 a, double s) { return D3{a.x * s, a.y * s, a.z * s}; }
 __device__ __forceinline__ D3 d3add(D3 a, D3 b) { return D3{a.x + b.x, a.y + b.y, a.z + b.z}; }
 
-// separation from atom `from` to atom `to`, nearest image
-__device__ __forceinline__ D3 mi(const D3* p, int from, int to, const double* L) {
+// separation from atom `from` to atom `to`, nearest image (the number of box
+// lengths in FP32: it is the same but for separations of half a box length)
+__device__ __forceinline__ D3 mi(const D3* p, int from, int to, const float* L) {
     D3 d = d3sub(p[to], p[from]);
-    d.x -= L[0] * rint(d.x / L[0]);
-    d.y -= L[1] * rint(d.y / L[1]);
-    d.z -= L[2] * rint(d.z / L[2]);
+    d.x = fma(-(double)L[0], (double)rintf((float)d.x / L[0]), d.x);
+    d.y = fma(-(double)L[1], (double)rintf((float)d.y / L[1]), d.y);
+    d.z = fma(-(double)L[2], (double)rintf((float)d.z / L[2]), d.z);
     return d;
 }
 
-__global__ void k_boresch(DevPtrs P) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= P.R) return;
-    const RepDev& R = P.reps[r];
-    if (R.boresch < 0) {
-        P.eb[r] = 0.0;
-        return;
+// cos and sin of the dihedral phi of b1, b2, b3 from phi = atan2(y, x),
+// x = n1.n2, y = |b2| b1.n2, without the angle itself (phi = 0 where it is
+// undefined, as atan2 has it)
+struct Dihedral {
+    D3 ga, gb, gc, gd;   // d phi / d x_a ... d x_d
+    double c, s;
+};
+__device__ __forceinline__ Dihedral dihedral(D3 b1, D3 b2, D3 b3) {
+    Dihedral d;
+    const D3 n1 = d3cross(b1, b2), n2 = d3cross(b2, b3);
+    const double l2 = d3dot(b2, b2), lb2 = sqrt(l2);
+    const double x = d3dot(n1, n2), y = lb2 * d3dot(b1, n2);
+    const double h2 = x * x + y * y, ih = h2 > 0.0 ? 1.0 / sqrt(h2) : 0.0;
+    d.c = h2 > 0.0 ? x * ih : (h2 == 0.0 ? 1.0 : h2);   // a NaN stays one
+    d.s = y * ih;
+    d.ga = d3scale(n1, -lb2 / d3dot(n1, n1));
+    d.gd = d3scale(n2, lb2 / d3dot(n2, n2));
+    const double il2 = 1.0 / l2, pp = d3dot(b1, b2) * il2, qq = d3dot(b3, b2) * il2;
+    d.gb = d3add(d3scale(d.ga, -(1.0 + pp)), d3scale(d.gd, qq));
+    d.gc = d3add(d3scale(d.ga, pp), d3scale(d.gd, -(1.0 + qq)));
+    return d;
+}
+
+__device__ __forceinline__ void add_force_d(const DevPtrs& P, int s, D3 g, double f) {
+    add_fixed(P.fx + s, to_fixed_d(f * g.x));
+    add_fixed(P.fy + s, to_fixed_d(f * g.y));
+    add_fixed(P.fz + s, to_fixed_d(f * g.z));
+}
+
+__device__ __forceinline__ D3 pos_d(const DevPtrs& P, int s) {
+    const float4 x = P.xq[s];
+    return D3{(double)x.x, (double)x.y, (double)x.z};
+}
+
+// One term of the Boresch restraint (0 distance P1-L1; 1, 2 angles P1-L1-L2 and
+// L1-P1-P2; 3-5 dihedrals P2-P1-L1-L2, P1-L1-L2-L3, L1-P1-P2-P3): adds its
+// forces times lambda_r and returns its energy. Anchors: 0 P1, 1 P2, 2 P3,
+// 3 L1, 4 L2, 5 L3.
+__device__ double boresch_term(const DevPtrs& P, const RepDev& R, const BoreschDev& B, int t) {
+    const float* L = R.box;
+    const double lr = R.dlam_r;
+    constexpr unsigned int ATOMS[6] = {0x30u, 0x430u, 0x103u, 0x4301u, 0x5430u, 0x2103u};
+    const unsigned int w = ATOMS[t];   // the term's anchors, first in the low four bits
+    const int n = t == 0 ? 2 : (t < 3 ? 3 : 4);
+    int sl[4];
+    D3 p[4];
+    for (int a = 0; a < 4; ++a) {
+        sl[a] = P.slot_of[R.atom_off + B.anc[a < n ? (w >> (4 * a)) & 15u : 0]];
+        p[a] = pos_d(P, sl[a]);
     }
-    const BoreschDev B = P.bor[R.boresch];
-    const double L[3] = {(double)R.box[0], (double)R.box[1], (double)R.box[2]};
-    D3 p[6];
-    int slot[6];
-    for (int a = 0; a < 6; ++a) {
-        slot[a] = P.slot_of[R.atom_off + B.anc[a]];
-        const float4 x = P.xq[slot[a]];
-        p[a] = D3{(double)x.x, (double)x.y, (double)x.z};
+    if (t == 0) {
+        const D3 d = mi(p, 0, 1, L);
+        const double rr = sqrt(d3dot(d, d)), dU = B.kr * (rr - B.r0);
+        if (lr != 0.0) {
+            const D3 g = d3scale(d, dU / rr);
+            add_force_d(P, sl[1], g, -lr);
+            add_force_d(P, sl[0], g, lr);
+        }
+        return 0.5 * B.kr * (rr - B.r0) * (rr - B.r0);
     }
-    // anchor slots: 0 P1, 1 P2, 2 P3, 3 L1, 4 L2, 5 L3
-    D3 grad[6];
-    for (int a = 0; a < 6; ++a) grad[a] = D3{0, 0, 0};
-    double U = 0.0;
-    {   // distance P1-L1
-        const D3 d = mi(p, 0, 3, L);
-        const double rr = sqrt(d3dot(d, d));
-        U += 0.5 * B.kr * (rr - B.r0) * (rr - B.r0);
-        const D3 g = d3scale(d, B.kr * (rr - B.r0) / rr);
-        grad[3] = d3add(grad[3], g);
-        grad[0] = d3sub(grad[0], g);
-    }
-    // angles (outer a, vertex b, outer c): P1-L1-L2 and L1-P1-P2
-    const int ang[2][3] = {{0, 3, 4}, {3, 0, 1}};
-    for (int t = 0; t < 2; ++t) {
-        const D3 u = mi(p, ang[t][1], ang[t][0], L), v = mi(p, ang[t][1], ang[t][2], L);
+    if (t < 3) {
+        const D3 u = mi(p, 1, 0, L), v = mi(p, 1, 2, L);
         const double lu = sqrt(d3dot(u, u)), lv = sqrt(d3dot(v, v));
         double c = d3dot(u, v) / (lu * lv);
         c = fmin(1.0, fmax(-1.0, c));
         const double th = acos(c);
         const double sn = sqrt(fmax(1.0 - c * c, 1e-300));
-        const double dU = B.kth * (th - B.th0[t]);
-        U += 0.5 * B.kth * (th - B.th0[t]) * (th - B.th0[t]);
-        // d theta / d u = -(v/|v| - cos u/|u|) / (|u| sin)
-        const D3 ga = d3scale(d3sub(d3scale(v, 1.0 / lv), d3scale(u, c / lu)), -1.0 / (lu * sn));
-        const D3 gc = d3scale(d3sub(d3scale(u, 1.0 / lu), d3scale(v, c / lv)), -1.0 / (lv * sn));
-        grad[ang[t][0]] = d3add(grad[ang[t][0]], d3scale(ga, dU));
-        grad[ang[t][2]] = d3add(grad[ang[t][2]], d3scale(gc, dU));
-        grad[ang[t][1]] = d3sub(grad[ang[t][1]], d3scale(d3add(ga, gc), dU));
-    }
-    // dihedrals a-b-c-d: P2-P1-L1-L2, P1-L1-L2-L3, L1-P1-P2-P3
-    const int dih[3][4] = {{1, 0, 3, 4}, {0, 3, 4, 5}, {3, 0, 1, 2}};
-    for (int t = 0; t < 3; ++t) {
-        const D3 b1 = mi(p, dih[t][0], dih[t][1], L);
-        const D3 b2 = mi(p, dih[t][1], dih[t][2], L);
-        const D3 b3 = mi(p, dih[t][2], dih[t][3], L);
-        const D3 n1 = d3cross(b1, b2), n2 = d3cross(b2, b3);
-        const double lb2 = sqrt(d3dot(b2, b2));
-        const double phi = atan2(lb2 * d3dot(b1, n2), d3dot(n1, n2));
-        const double dU = B.kph * sin(phi - B.ph0[t]);
-        U += B.kph * (1.0 - cos(phi - B.ph0[t]));
-        const D3 ga = d3scale(n1, -lb2 / d3dot(n1, n1));
-        const D3 gd = d3scale(n2, lb2 / d3dot(n2, n2));
-        const double pp = d3dot(b1, b2) / (lb2 * lb2), qq = d3dot(b3, b2) / (lb2 * lb2);
-        const D3 gb = d3add(d3scale(ga, -(1.0 + pp)), d3scale(gd, qq));
-        const D3 gc = d3add(d3scale(ga, pp), d3scale(gd, -(1.0 + qq)));
-        grad[dih[t][0]] = d3add(grad[dih[t][0]], d3scale(ga, dU));
-        grad[dih[t][1]] = d3add(grad[dih[t][1]], d3scale(gb, dU));
-        grad[dih[t][2]] = d3add(grad[dih[t][2]], d3scale(gc, dU));
-        grad[dih[t][3]] = d3add(grad[dih[t][3]], d3scale(gd, dU));
-    }
-    const double lr = R.dlam_r;
-    if (lr != 0.0) {
-        for (int a = 0; a < 6; ++a) {
-            add_fixed(P.fx + slot[a], to_fixed_d(-lr * grad[a].x));
-            add_fixed(P.fy + slot[a], to_fixed_d(-lr * grad[a].y));
-            add_fixed(P.fz + slot[a], to_fixed_d(-lr * grad[a].z));
+        const double dU = B.kth * (th - B.th0[t - 1]);
+        if (lr != 0.0) {
+            // d theta / d u = -(v/|v| - cos u/|u|) / (|u| sin)
+            const D3 ga = d3scale(d3sub(d3scale(v, 1.0 / lv), d3scale(u, c / lu)), -1.0 / (lu * sn));
+            const D3 gc = d3scale(d3sub(d3scale(u, 1.0 / lu), d3scale(v, c / lv)), -1.0 / (lv * sn));
+            add_force_d(P, sl[0], ga, -lr * dU);
+            add_force_d(P, sl[2], gc, -lr * dU);
+            add_force_d(P, sl[1], d3add(ga, gc), lr * dU);
         }
+        return 0.5 * B.kth * (th - B.th0[t - 1]) * (th - B.th0[t - 1]);
     }
-    if (!isfinite(U)) set_err(P.cnt, ERRB_NONFINITE, r);
-    P.eb[r] = U;
+    // U = k [1 - cos(phi - phi0)], the difference's cosine and sine by addition
+    const Dihedral d = dihedral(mi(p, 0, 1, L), mi(p, 1, 2, L), mi(p, 2, 3, L));
+    const double c0 = B.cph0[t - 3], s0 = B.sph0[t - 3];
+    if (lr != 0.0) {
+        const double f = -lr * B.kph * (d.s * c0 - d.c * s0);
+        add_force_d(P, sl[0], d.ga, f);
+        add_force_d(P, sl[1], d.gb, f);
+        add_force_d(P, sl[2], d.gc, f);
+        add_force_d(P, sl[3], d.gd, f);
+    }
+    return B.kph * (1.0 - (d.c * c0 + d.s * s0));
 }
 
-// U = s sum_t k_t [1 + cos(n_t phi_t - phi0_t)], s = lambda_v (annihilation)
-// or 1 (decoupling); phi from b1 = x_b - x_a, b2 = x_c - x_b, b3 = x_d - x_c
-// (nearest images) as atan2(|b2| b1.(b2 x b3), (b1 x b2).(b2 x b3)). The
-// gradient: d phi/d x_a = -|b2| n1/|n1|^2, d phi/d x_d = |b2| n2/|n2|^2 and the
-// inner atoms from those with the projections b1.b2/|b2|^2 and b3.b2/|b2|^2.
-// The unscaled sum goes to EA_TORS, and (annihilation) to dU/dlambda_v.
-__global__ void __launch_bounds__(128) k_torsions(DevPtrs P) {
-    const int rep = blockIdx.y;
-    const RepDev& R = P.reps[rep];
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    double e = 0.0;
-    if (t < R.n_tors) {
-        const int4 q = P.sys_tors[R.tors_off + t];
-        const dbl4 prm = P.sys_torsp[R.tors_off + t];
-        const int sl[4] = {P.slot_of[R.atom_off + q.x], P.slot_of[R.atom_off + q.y],
-                           P.slot_of[R.atom_off + q.z], P.slot_of[R.atom_off + q.w]};
-        D3 p[4];
-        for (int a = 0; a < 4; ++a) {
-            const float4 x = P.xq[sl[a]];
-            p[a] = D3{(double)x.x, (double)x.y, (double)x.z};
-        }
-        const double L[3] = {(double)R.box[0], (double)R.box[1], (double)R.box[2]};
-        const D3 b1 = mi(p, 0, 1, L), b2 = mi(p, 1, 2, L), b3 = mi(p, 2, 3, L);
-        const D3 n1 = d3cross(b1, b2), n2 = d3cross(b2, b3);
-        const double lb2 = sqrt(d3dot(b2, b2));
-        const double phi = atan2(lb2 * d3dot(b1, n2), d3dot(n1, n2));
-        const double arg = prm.y * phi - prm.z;
-        e = prm.x * (1.0 + cos(arg));
-        const bool ann = P.ligand_mode == 0;
-        const double s = ann ? R.dlam_v : 1.0;
-        // dU/dphi of the state
-        const double dU = -s * prm.x * prm.y * sin(arg);
-        if (dU != 0.0) {
-            const D3 ga = d3scale(n1, -lb2 / d3dot(n1, n1));
-            const D3 gd = d3scale(n2, lb2 / d3dot(n2, n2));
-            const double pp = d3dot(b1, b2) / (lb2 * lb2), qq = d3dot(b3, b2) / (lb2 * lb2);
-            const D3 g[4] = {ga, d3add(d3scale(ga, -(1.0 + pp)), d3scale(gd, qq)),
-                             d3add(d3scale(ga, pp), d3scale(gd, -(1.0 + qq))), gd};
-            for (int a = 0; a < 4; ++a) {
-                add_fixed(P.fx + sl[a], to_fixed_d(-dU * g[a].x));
-                add_fixed(P.fy + sl[a], to_fixed_d(-dU * g[a].y));
-                add_fixed(P.fz + sl[a], to_fixed_d(-dU * g[a].z));
-            }
-        }
+// One torsion k [1 + cos(n phi - phi0)], scaled by s = lambda_v (annihilation) or
+// 1 (decoupling): adds its forces and returns its unscaled energy. cos and sin of
+// n phi (n <= 6) by complex powers, of the difference by addition.
+__device__ double torsion_term(const DevPtrs& P, const RepDev& R, int t) {
+    const int4 q = P.sys_tors[R.tors_off + t];
+    const dbl4 prm = P.sys_torsp[R.tors_off + t];   // k, n, cos phi0, sin phi0
+    const int sl[4] = {P.slot_of[R.atom_off + q.x], P.slot_of[R.atom_off + q.y],
+                       P.slot_of[R.atom_off + q.z], P.slot_of[R.atom_off + q.w]};
+    const D3 p[4] = {pos_d(P, sl[0]), pos_d(P, sl[1]), pos_d(P, sl[2]), pos_d(P, sl[3])};
+    const float* L = R.box;
+    const Dihedral d = dihedral(mi(p, 0, 1, L), mi(p, 1, 2, L), mi(p, 2, 3, L));
+    double cn = d.c, sn = d.s;
+    for (int m = (int)prm.y; m > 1; --m) {
+        const double c = cn * d.c - sn * d.s;
+        sn = sn * d.c + cn * d.s;
+        cn = c;
     }
-    __shared__ double s_e[4];
-    double de = e;
-    for (int o = 16; o > 0; o >>= 1) de += __shfl_xor_sync(FULL, de, o);
-    if ((threadIdx.x & 31) == 0) s_e[threadIdx.x >> 5] = de;
+    const double s = P.ligand_mode == 0 ? R.dlam_v : 1.0;
+    const double f = s * prm.x * prm.y * (sn * prm.z - cn * prm.w);   // -dU/dphi
+    if (f != 0.0) {
+        add_force_d(P, sl[0], d.ga, f);
+        add_force_d(P, sl[1], d.gb, f);
+        add_force_d(P, sl[2], d.gc, f);
+        add_force_d(P, sl[3], d.gd, f);
+    }
+    return prm.x * (1.0 + (cn * prm.z + sn * prm.w));
+}
+
+// The FP64 bonded terms of a replica (block): warps 0-2 take its torsions, warp 3
+// the angles and the dihedrals of its Boresch restraint, warp 2 the restraint's
+// distance. Bound by FP64 latency (63 issue cycles per warp instruction on this
+// chip), so the restraint's terms run on lanes of their own and no term calls a
+// trigonometric function but acos: 54 us (restraint, one thread per replica) and
+// 17 us (torsions, atan2 + cos + sin) in two launches before, 9 us together now
+// (24 windows of 25k atoms).
+__global__ void __launch_bounds__(128) k_restraints(DevPtrs P) {
+    const int rep = blockIdx.x;
+    const RepDev& R = P.reps[rep];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double s_b[6], s_t[3];
+    double et = 0.0;
+    if (w < 3)
+        for (int t = threadIdx.x; t < R.n_tors; t += 96) et += torsion_term(P, R, t);
+    if (R.boresch >= 0) {
+        const BoreschDev& B = P.bor[R.boresch];
+        if (w == 3 && lane < 5) s_b[lane + 1] = boresch_term(P, R, B, lane + 1);
+        if (w == 2 && lane == 31) s_b[0] = boresch_term(P, R, B, 0);
+    }
+    __syncwarp();
+    for (int o = 16; o > 0; o >>= 1) et += __shfl_xor_sync(FULL, et, o);
+    if (w < 3 && lane == 0) s_t[w] = et;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double tt = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tt += s_e[w];
-        if (!isfinite(tt)) set_err(P.cnt, ERRB_NONFINITE, rep);
+        const double U = R.boresch < 0 ? 0.0 : s_b[0] + s_b[1] + s_b[2] + s_b[3] + s_b[4] + s_b[5];
+        P.eb[rep] = U;
+        const double tt = s_t[0] + s_t[1] + s_t[2];
+        if (!isfinite(tt) || !isfinite(U)) set_err(P.cnt, ERRB_NONFINITE, rep);
         if (tt != 0.0) {
+            // the unscaled sum, and (annihilation) dU/dlambda_v
             add_fixed(P.eacc + (size_t)rep * EA_N + EA_TORS, to_fixed_d(tt));
             if (P.ligand_mode == 0) add_fixed(P.eacc + (size_t)rep * EA_N + EA_DUDLV, to_fixed_d(tt));
         }
@@ -827,12 +842,6 @@ void launch_bonds(const DevPtrs& P, cudaStream_t s, int precision, bool energy) 
     }
 }
 
-void launch_torsions(const DevPtrs& P, cudaStream_t s, int max_tors) {
-    if (max_tors <= 0) return;
-    dim3 grid((max_tors + 127) / 128, P.R);
-    k_torsions<<<grid, 128, 0, s>>>(P);
-}
-
 void launch_aw_refresh(const DevPtrs& P, cudaStream_t s) {
     k_aw_refresh<<<P.R, 32, 0, s>>>(P);
 }
@@ -842,8 +851,8 @@ void launch_aw_sums(const DevPtrs& P, cudaStream_t s, int max_aw) {
     k_aw_sums<<<dim3(max_aw, P.R), 128, 0, s>>>(P);
 }
 
-void launch_boresch(const DevPtrs& P, cudaStream_t s) {
-    k_boresch<<<(P.R + 63) / 64, 64, 0, s>>>(P);
+void launch_restraints(const DevPtrs& P, cudaStream_t s) {
+    k_restraints<<<P.R, 128, 0, s>>>(P);
 }
 
 void launch_finalize(const DevPtrs& P, cudaStream_t s) {

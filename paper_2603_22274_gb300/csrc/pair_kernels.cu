@@ -5,11 +5,9 @@
 //   cutoff, over the inner list of j rows. A warp owns one i-cluster (8 atoms,
 //   held in shared memory) and walks its rows 32 at a time, a lane per row:
 //   the lane loads the row's j atom once and evaluates it against the i atoms
-//   the row covers (all 8 of a full row; atoms 0-3 or 4-7 of a half row, the
-//   rows being ordered full | lower half | upper half so that most rounds
-//   skip the unused half block for the whole warp); its j force goes to the
-//   64-bit fixed-point accumulators once per row and the i forces stay in
-//   registers until the item ends. FP32 forces: the Coulomb force is
+//   the row covers (all 8 of a full row; atoms 0-3 or 4-7 of a half row); its j
+//   force goes to the 64-bit fixed-point accumulators once per row and the i
+//   forces stay in registers until the item ends. FP32 forces: the Coulomb force is
 //   qq G(r) / r^3 with G from a quadratic table in r held in shared memory
 //   (ewald_G); FP32 energies (energy steps only) use correctly rounded
 //   arithmetic and erfcf/expf; FP64 uses erfc/exp.
@@ -144,6 +142,7 @@ __device__ __forceinline__ const RowItem& row_item(const DevPtrs& P, int it) {
 }
 
 // ------------------------------------------------------------------ env pair
+// (a pair that is not kept adds exact zeros)
 template <typename T, bool ENERGY>
 __device__ __forceinline__ void pair_env(const Atom<T>& ai, const Atom<T>& aj, bool keep,
                                          T3<T>& fi, T3<T>& fj, T& elj, T& ec, const KC<T>& K) {
@@ -272,14 +271,13 @@ __device__ __forceinline__ int warp_sum_24(T (&v)[24], int lane) {
 
 // ------------------------------------------------------------------ env rows
 // Lane per j row: lane l of a warp takes row k0 + l of its item, loads the
-// row's j atom once and evaluates it against the i atoms the row covers (all
-// 8 for a full row, atoms 0-3 or 4-7 for a half row), read as broadcasts from
-// the warp's copy of the i-cluster in shared memory. The j force stays in the
-// lane and goes to the fixed-point accumulators once per row; the i forces
-// stay in registers (8 atoms x 3) until the item ends and are then summed
-// over the warp. A block of eight pairs per row gives every lane eight
-// independent chains of arithmetic; a pair block no lane of the warp needs
-// (a round of half rows of one kind) is skipped.
+// row's j atom once and evaluates it against the cluster's 8 i atoms, read as
+// broadcasts from the warp's copy of the i-cluster in shared memory. The j force
+// stays in the lane and goes to the fixed-point accumulators once per row; the i
+// forces stay in registers (8 atoms x 3) until the item ends and are then summed
+// over the warp. Rounds of 32 full rows evaluate eight pairs per lane without a
+// check; the last one or two rounds of an item (the remaining full rows, rows with
+// only atoms 0-3 or 4-7 in range, masked rows, idle lanes) check each pair.
 constexpr int ENV_WARPS_MAX = 8;
 
 // one i atom in shared memory: x, y, z, q sqrt(ke), sigma/2, 2 sqrt(eps), -, -
@@ -288,7 +286,7 @@ __device__ __forceinline__ Atom<T> ld_iatom(const T* p);
 template <>
 __device__ __forceinline__ Atom<float> ld_iatom<float>(const float* p) {
     const float4 a = reinterpret_cast<const float4*>(p)[0];
-    const float4 b = reinterpret_cast<const float4*>(p)[1];
+    const float2 b = reinterpret_cast<const float2*>(p)[2];
     return Atom<float>{a.x, a.y, a.z, a.w, b.x, b.y};
 }
 template <>
@@ -304,165 +302,195 @@ __device__ __forceinline__ void st_iatom(T* p, const Atom<T>& a) {
     p[6] = (T)0; p[7] = (T)0;
 }
 
-// round kinds (warp-uniform): every lane a full row; every lane a row with
-// only atoms 0-3 (LO) or only atoms 4-7 (HI) in range; anything else (mixed
-// kinds, masked rows, idle lanes) with per-pair checks
-enum : int { RM_FULL = 0, RM_LO = 1, RM_HI = 2, RM_MIXED = 3 };
+// adds a force component to an accumulator unless it is zero (no pair in range)
+template <typename T>
+__device__ __forceinline__ void red_nonzero(long long* p, T f) {
+    const long long v = sizeof(T) == 8 ? to_fixed_d((double)f) : to_fixed((float)f);
+    if (f != (T)0) add_fixed(p, v);
+}
 
-// One row of a lane: its j atom (already shifted) against the i atoms of the
-// active halves, minus the excluded ones (em) of a masked row; the j force
-// goes to the accumulators.
-template <typename T, bool ENERGY, int MODE>
-__device__ __forceinline__ void env_row(const DevPtrs& P, const KC<T>& K, const T* s_ia, int ja,
-                                        const Atom<T>& aj, bool act_lo, bool act_hi,
-                                        unsigned int em, T3<T> (&fi)[CL], double& elj_d,
+// One row of a lane against the i atoms; CHECK: minus those in `em`.
+template <typename T, bool ENERGY, bool CHECK>
+__device__ __forceinline__ void env_row(const DevPtrs& P, const KC<T>& K, const T* s_ia,
+                                        const float4* sh, unsigned int word, unsigned int em,
+                                        const Atom<T>& aj, T3<T> (&fi)[CL], double& elj_d,
                                         double& ec_d) {
+    // the j atom relative to the cluster's reference atom c, (x_j + u) - v
+    // with (u, v) from the row's image code
+    const int code = (int)(word >> ROW_SLOT_BITS);
+    const float4 u = sh[code], v = sh[32 + code];
+    Atom<T> a = aj;
+    a.x = ((T)aj.x + (T)u.x) - (T)v.x;
+    a.y = ((T)aj.y + (T)u.y) - (T)v.y;
+    a.z = ((T)aj.z + (T)u.z) - (T)v.z;
     T3<T> fj{(T)0, (T)0, (T)0};
     T elj = 0, ec = 0;
-    constexpr int i0 = MODE == RM_HI ? 4 : 0, i1 = MODE == RM_LO ? 4 : CL;
 #pragma unroll
-    for (int ii = i0; ii < i1; ++ii) {
-        if (MODE != RM_MIXED || ((ii < 4 ? act_lo : act_hi) && !((em >> ii) & 1u)))
-            pair_env<T, ENERGY>(ld_iatom<T>(s_ia + ii * 8), aj, true, fi[ii], fj, elj, ec, K);
+    for (int ii = 0; ii < CL; ++ii) {
+        // (FP64: skipped rather than evaluated and dropped)
+        if (CHECK && sizeof(T) == 8 && ((em >> ii) & 1u)) continue;
+        pair_env<T, ENERGY>(ld_iatom<T>(s_ia + ii * 8), a, !(CHECK && ((em >> ii) & 1u)), fi[ii], fj,
+                            elj, ec, K);
     }
     if (ENERGY) {
         elj_d += (double)elj;
         ec_d += (double)ec;
     }
-    if (MODE != RM_MIXED || act_lo || act_hi) {
-        const bool dbl = sizeof(T) == 8;
-        if (fj.x != (T)0) add_fixed(P.fx + ja, dbl ? to_fixed_d((double)fj.x) : to_fixed((float)fj.x));
-        if (fj.y != (T)0) add_fixed(P.fy + ja, dbl ? to_fixed_d((double)fj.y) : to_fixed((float)fj.y));
-        if (fj.z != (T)0) add_fixed(P.fz + ja, dbl ? to_fixed_d((double)fj.z) : to_fixed((float)fj.z));
-    }
+    const int ja = (int)(word & ROW_SLOT_MASK);
+    red_nonzero<T>(P.fx + ja, fj.x);
+    red_nonzero<T>(P.fy + ja, fj.y);
+    red_nonzero<T>(P.fz + ja, fj.z);
 }
 
-// All rows of one item, 32 per round: row k < n_plain is plain row k (runs:
-// full | atoms 0-3 only | atoms 4-7 only), row k >= n_plain masked row
-// k - n_plain, so an item ends in one partly filled round. The next round's
-// row word and j atom are loaded before the current round is computed (word,
-// then atom: the loads depend on each other).
-template <typename T, bool ENERGY>
-__device__ __forceinline__ void env_rows(const DevPtrs& P, const KC<T>& K, const RepDev& R,
-                                         const RowItem& I, const float4* sh, const T* s_ia,
-                                         int lane, T3<T> (&fi)[CL], double& elj, double& ec) {
-    const int n_full = I.cnt & 0xFFFF, n_lo_end = n_full + I.n_lo;
-    const int n_plain = n_lo_end + I.n_hi, n = n_plain + (I.cnt >> 16);
-    if (n <= 0) return;
-    auto fetch = [&](int k, unsigned int& word, unsigned int& em) {
-        const int kk = k < n ? k : n - 1;
-        if (kk < n_plain) {
-            word = P.rows[I.r_begin + (unsigned int)kk];
-            em = 0u;
-        } else {
-            const int2 xr = P.xrows[I.x_begin + (kk - n_plain)];
-            word = (unsigned int)xr.x;
-            em = (unsigned int)xr.y;
-        }
-    };
-    unsigned int word, em;
-    fetch(lane, word, em);
-    Atom<T> aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
-    for (int k0 = 0; k0 < n; k0 += 32) {
-        const int k = k0 + lane;
-        unsigned int word_n = word, em_n = em;
-        Atom<T> aj_n = aj;
-        if (k0 + 32 < n) {   // warp-uniform
-            fetch(k + 32, word_n, em_n);
-            aj_n = load_atom<T>(P, (int)(word_n & ROW_SLOT_MASK), R, K);
-        }
-        // the j atom relative to the cluster's reference atom c, (x_j + u) - v
-        // with (u, v) from the row's image code (see the table below)
-        const int code = (int)(word >> ROW_SLOT_BITS);
-        const float4 u = sh[code], v = sh[32 + code];
-        Atom<T> a = aj;
-        a.x = ((T)aj.x + (T)u.x) - (T)v.x;
-        a.y = ((T)aj.y + (T)u.y) - (T)v.y;
-        a.z = ((T)aj.z + (T)u.z) - (T)v.z;
-        const int ja = (int)(word & ROW_SLOT_MASK);
-        // the round's kind (warp-uniform)
-        if (k0 + 32 <= n_full) {
-            env_row<T, ENERGY, RM_FULL>(P, K, s_ia, ja, a, true, true, 0u, fi, elj, ec);
-        } else if (k0 >= n_full && k0 + 32 <= n_lo_end) {
-            env_row<T, ENERGY, RM_LO>(P, K, s_ia, ja, a, true, false, 0u, fi, elj, ec);
-        } else if (k0 >= n_lo_end && k0 + 32 <= n_plain) {
-            env_row<T, ENERGY, RM_HI>(P, K, s_ia, ja, a, false, true, 0u, fi, elj, ec);
-        } else {
-            const bool valid = k < n;
-            const bool masked = k >= n_plain;
-            const bool act_lo = valid && (masked || k < n_lo_end);
-            const bool act_hi = valid && (masked || k < n_full || k >= n_lo_end);
-            env_row<T, ENERGY, RM_MIXED>(P, K, s_ia, ja, a, act_lo, act_hi, em, fi, elj, ec);
-        }
-        word = word_n;
-        em = em_n;
-        aj = aj_n;
+// row k of an item (I: the words of a RowItem) beyond its full rounds: plain
+// rows (full | atoms 0-3 only | atoms 4-7 only), then masked rows; the i atoms
+// that it must not meet (all of them past the last row)
+__device__ __forceinline__ void env_tail_row(const DevPtrs& P, const volatile int* I, int k,
+                                             unsigned int& word, unsigned int& em) {
+    const int n_full = I[3] & 0xFFFF, n_lo_end = n_full + I[4], n_plain = n_lo_end + I[5],
+              n = n_plain + (I[3] >> 16);
+    const int kk = min(k, n - 1);
+    if (kk < n_plain) {
+        word = P.rows[(unsigned int)I[1] + (unsigned int)kk];
+        em = kk < n_full ? 0u : (kk < n_lo_end ? 0xF0u : 0x0Fu);
+    } else {
+        const int2 xr = P.xrows[I[2] + (kk - n_plain)];
+        word = (unsigned int)xr.x;
+        em = (unsigned int)xr.y;
     }
+    if (k >= n) em = 0xFFu;
 }
 
-template <typename T, bool ENERGY>
-__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : (ENERGY ? 3 : 4)) k_env_rows(DevPtrs P) {
+// A warp's first item is its own index, dealt over the blocks, so that a small
+// system needs no claims (4,864 warps claiming one counter take 3 us) and its
+// idle blocks leave at once; later items are claimed, up to four at a time (one
+// claim per item serialised on the counter: +0.5 ms per launch on the
+// 1,152-window batch), fewer when there are few items per warp. MINB: blocks of
+// 256 threads per SM that the registers allow (4: 64 registers, for many items
+// per warp; fewer for small systems, see env_small).
+//
+// The item and the claim counters live in shared memory (volatile: read again
+// where they are needed), so that 64 registers hold the round loop: with them in
+// registers it spilled inside the loop, which cost more than the atom of the
+// next round loaded ahead gained (24 x 25k atoms: 429 us with the prefetch, 472
+// with this claim scheme in registers too, 400 as it is).
+template <typename T, bool ENERGY, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    KC<T> K = make_kc<T>(P);
     __shared__ float4 s_ewtab[sizeof(T) == 4 ? EW_NT : 1];
     // per warp and image code: u (0-26) and v (32-58) of the shifted j atom
     // relative to the i-cluster's reference atom
     __shared__ float4 s_shift[ENV_WARPS_MAX][64];
     __shared__ __align__(16) T s_iat[ENV_WARPS_MAX][CL * 8];
-    if constexpr (sizeof(T) == 4) {
-        for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_ewtab[i] = P.ewtab[i];
+    __shared__ int s_item[ENV_WARPS_MAX][8];   // the warp's RowItem
+    __shared__ int s_next[ENV_WARPS_MAX][2];   // its next item, end of the claimed ones
+    volatile int* const I = s_item[w];
+    volatile int* const N = s_next[w];
+    KC<T> K = make_kc<T>(P);
+    {
+        const int n_items = P.ritem_pref[P.R];
+        if ((int)blockIdx.x >= n_items) return;   // no warp of this block has an item
+        if constexpr (sizeof(T) == 4) {
+            for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_ewtab[i] = P.ewtab[i];
+            K.tab = s_ewtab;
+        }
+        if (lane == 0) {
+            N[0] = w * (int)gridDim.x + (int)blockIdx.x;
+            N[1] = min(N[0] + 1, n_items);
+        }
         __syncthreads();
-        K.tab = s_ewtab;
     }
-    float4* sh = s_shift[w];
-    T* s_ia = s_iat[w];
-    const int n_items = P.ritem_pref[P.R];
-    // items are claimed up to four at a time (one claim per item serialised on
-    // the counter: +0.5 ms per launch on the 1,152-window batch), fewer when
-    // there are few items per warp
-    const int chunk = max(1, min(4, n_items / ((int)(gridDim.x * (blockDim.x >> 5)) * 8)));
-    int it_next = 0, it_end = 0;
+    float4* const sh = s_shift[w];
+    T* const s_ia = s_iat[w];
     for (;;) {
-        if (it_next >= it_end) {
-            int c0 = 0;
-            if (lane == 0) c0 = atomicAdd(&P.cnt->env_next, chunk);
-            c0 = __shfl_sync(FULL, c0, 0);
-            if (c0 >= n_items) break;
-            it_next = c0;
-            it_end = min(c0 + chunk, n_items);
+        {
+            __syncwarp();
+            int it = N[0];
+            const int it_end = N[1];
+            __syncwarp();
+            if (it >= it_end) {
+                const int nw = (int)(gridDim.x * (blockDim.x >> 5)), n_items = P.ritem_pref[P.R];
+                if (nw >= n_items) break;
+                const int chunk = max(1, min(4, n_items / (nw * 8)));
+                if (lane == 0) it = nw + atomicAdd(&P.cnt->env_next, chunk);
+                it = __shfl_sync(FULL, it, 0);
+                if (it >= n_items) break;
+                if (lane == 0) N[1] = min(it + chunk, n_items);
+            }
+            if (lane == 0) N[0] = it + 1;
+            const RowItem& item = row_item(P, it);
+            if (lane < 8) I[lane] = reinterpret_cast<const int*>(&item)[lane];
+            __syncwarp();
+            // image shifts of this replica's box, by code; the i-cluster's atoms
+            // relative to its first atom (the reference c; same cluster: exact)
+            // x_j + s - c for image shift s is evaluated as (x_j + u) - v with
+            // u = s - c, v = 0 where s > 0 (then c lies near the box length, and
+            // s - c is exact) and u = s, v = c otherwise (x_j + s is exact where
+            // s < 0, x_j lying near the box length): no box-sized sum is rounded
+            const RepDev& R = P.reps[P.rep_of_cl[I[0]]];
+            const float4 c = P.xq[I[0] * CL];
+            if (lane < 27) {
+                const float sx = (float)(lane % 3 - 1) * R.box[0],
+                            sy = (float)((lane / 3) % 3 - 1) * R.box[1],
+                            sz = (float)(lane / 9 - 1) * R.box[2];
+                sh[lane] = make_float4(sx > 0.f ? sx - c.x : sx, sy > 0.f ? sy - c.y : sy,
+                                       sz > 0.f ? sz - c.z : sz, 0.f);
+                sh[32 + lane] = make_float4(sx > 0.f ? 0.f : c.x, sy > 0.f ? 0.f : c.y,
+                                            sz > 0.f ? 0.f : c.z, 0.f);
+            }
+            if (lane < CL) {
+                Atom<T> ai = load_atom<T>(P, I[0] * CL + lane, R, K);
+                ai.x -= (T)c.x;
+                ai.y -= (T)c.y;
+                ai.z -= (T)c.z;
+                st_iatom<T>(s_ia + lane * 8, ai);
+            }
+            __syncwarp();
         }
-        const int it = it_next++;
-        const RowItem I = row_item(P, it);
-        const int rep = P.rep_of_cl[I.c];
-        const RepDev& R = P.reps[rep];
-        // image shifts of this replica's box, by code; the i-cluster's atoms
-        // relative to its first atom (the reference c; same cluster: exact)
-        // x_j + s - c for image shift s is evaluated as (x_j + u) - v with
-        // u = s - c, v = 0 where s > 0 (then c lies near the box length, and
-        // s - c is exact) and u = s, v = c otherwise (x_j + s is exact where
-        // s < 0, x_j lying near the box length): no box-sized sum is rounded
-        const float4 c = P.xq[I.c * CL];
-        if (lane < 27) {
-            const float sx = (float)(lane % 3 - 1) * R.box[0], sy = (float)((lane / 3) % 3 - 1) * R.box[1],
-                        sz = (float)(lane / 9 - 1) * R.box[2];
-            sh[lane] = make_float4(sx > 0.f ? sx - c.x : sx, sy > 0.f ? sy - c.y : sy,
-                                   sz > 0.f ? sz - c.z : sz, 0.f);
-            sh[32 + lane] = make_float4(sx > 0.f ? 0.f : c.x, sy > 0.f ? 0.f : c.y,
-                                        sz > 0.f ? 0.f : c.z, 0.f);
-        }
-        if (lane < CL) {
-            Atom<T> ai = load_atom<T>(P, I.c * CL + lane, R, K);
-            ai.x -= (T)c.x;
-            ai.y -= (T)c.y;
-            ai.z -= (T)c.z;
-            st_iatom<T>(s_ia + lane * 8, ai);
-        }
-        __syncwarp();
         T3<T> fi[CL];
 #pragma unroll
         for (int ii = 0; ii < CL; ++ii) fi[ii] = T3<T>{(T)0, (T)0, (T)0};
         double elj = 0.0, ec = 0.0;
-        env_rows<T, ENERGY>(P, K, R, I, sh, s_ia, lane, fi, elj, ec);
+        // FP64 parameters are looked up per replica
+        const RepDev& R = P.reps[sizeof(T) == 8 ? P.rep_of_cl[I[0]] : 0];
+        {
+            // full rounds: the next round's row word is loaded a round ahead, its atom
+            // is not (the other warps cover that latency at fewer registers) unless
+            // there are no other warps
+            int nf = (I[3] & 0xFFFF) >> 5;
+            const unsigned int* rp = P.rows + ((unsigned int)I[1] + (unsigned int)lane);
+            unsigned int word = nf > 0 ? *rp : 0u;
+            if (MINB == 1) {
+                Atom<T> aj{};
+                if (nf > 0) aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
+                for (; nf > 0; --nf) {
+                    rp += 32;
+                    unsigned int word_n = word;
+                    Atom<T> aj_n = aj;
+                    if (nf > 1) {
+                        word_n = *rp;
+                        aj_n = load_atom<T>(P, (int)(word_n & ROW_SLOT_MASK), R, K);
+                    }
+                    env_row<T, ENERGY, false>(P, K, s_ia, sh, word, 0u, aj, fi, elj, ec);
+                    word = word_n;
+                    aj = aj_n;
+                }
+            } else {
+                for (; nf > 0; --nf) {
+                    rp += 32;
+                    const unsigned int word_n = nf > 1 ? *rp : 0u;
+                    const Atom<T> aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
+                    env_row<T, ENERGY, false>(P, K, s_ia, sh, word, 0u, aj, fi, elj, ec);
+                    word = word_n;
+                }
+            }
+        }
+        for (int k0 = (I[3] & 0xFFFF) & ~31; k0 < (I[3] & 0xFFFF) + I[4] + I[5] + (I[3] >> 16); k0 += 32) {
+            unsigned int word, em;
+            env_tail_row(P, I, k0 + lane, word, em);
+            const Atom<T> aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
+            env_row<T, ENERGY, true>(P, K, s_ia, sh, word, em, aj, fi, elj, ec);
+        }
         // i forces: the 24 values 3 ii + c summed over the warp (transposed);
         // value v ends on the four lanes of group v / 3, and the lane with
         // lane % 4 == v % 3 < 3 writes it
@@ -477,19 +505,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : (ENERGY ? 3 : 4)) k_
         if ((lane & 3) < 3 && v[0] != (T)0) {
             const int c = vi % 3;
             long long* d = c == 0 ? P.fx : (c == 1 ? P.fy : P.fz);
-            add_fixed(d + I.c * CL + vi / 3,
+            add_fixed(d + I[0] * CL + vi / 3,
                       (sizeof(T) == 4) ? to_fixed((float)v[0]) : to_fixed_d((double)v[0]));
         }
         if (ENERGY) {
             const double sl = warp_sum<double>(elj);
             const double sc = warp_sum<double>(ec);
             if (lane == 0) {
+                const int rep = P.rep_of_cl[I[0]];
                 if (!isfinite(sl) || !isfinite(sc)) set_err(P.cnt, ERRB_NONFINITE, rep);
                 add_fixed(P.eacc + (size_t)rep * EA_N + EA_ENV_LJ, to_fixed_d(sl));
                 add_fixed(P.eacc + (size_t)rep * EA_N + EA_ENV_C, to_fixed_d(sc));
             }
         }
-        __syncwarp();
     }
 }
 
@@ -574,16 +602,37 @@ __device__ __forceinline__ LigState<double> lig_state<double>(const DevPtrs& P, 
     return S;
 }
 
+// The entries of a ligand item, 32 at a time: lane l holds entry base + l (and
+// its exclusion mask), so that the loop over entries takes them by shuffles and
+// the j atoms of the next entry can be loaded ahead.
+struct LigEntries {
+    int2 e;
+    unsigned long long m;
+    __device__ __forceinline__ void load(const DevPtrs& P, const Item& I, int base, int lane) {
+        const int t = base + lane;
+        e = make_int2(0, 0);
+        m = 0ull;
+        if (t < I.e_cnt) {
+            e = P.entries[I.e_begin + t];
+        } else if (t < I.e_cnt + I.x_cnt) {
+            const int k = I.x_begin + (t - I.e_cnt);
+            e = P.xentries[k];
+            m = P.xmasks[(size_t)k * GMAX];
+        }
+    }
+};
+
+// Latency bound (a few hundred pairs per window): a warp's first item is its own
+// index (no claim), the entries are loaded together and the j atoms one entry
+// ahead.
 template <typename T, bool ENERGY>
 __global__ void __launch_bounds__(128) k_lig(DevPtrs P) {
     const int lane = threadIdx.x & 31, jj = lane & 7, ii = lane >> 3;
     const KC<T> K = make_kc<T>(P);
     const int n_items = P.ilig_pref[P.R];
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = atomicAdd(&P.cnt->lig_next, 1);
-        it = __shfl_sync(FULL, it, 0);
-        if (it >= n_items) break;
+    const int nw = (int)gridDim.x * 4;
+    int it = (threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
+    while (it < n_items) {
         const Item I = P.items_lig[region_index(P.ilig_pref, P.ilig_base, P.R, it)];
         const RepDev& R = P.reps[I.rep];
         const int a0 = I.c0 * CL + ii;
@@ -596,17 +645,23 @@ __global__ void __launch_bounds__(128) k_lig(DevPtrs P) {
         T3<T> fi0{(T)0, (T)0, (T)0}, fi1{(T)0, (T)0, (T)0};
         double acc[6] = {0, 0, 0, 0, 0, 0};
         const int ntot = I.e_cnt + I.x_cnt;
+        LigEntries L;
+        Atom<T> aj_n{};
         for (int t = 0; t < ntot; ++t) {
-            const bool xm = t >= I.e_cnt;
-            const int k = xm ? I.x_begin + (t - I.e_cnt) : I.e_begin + t;
-            const int2 e = xm ? P.xentries[k] : P.entries[k];
-            const unsigned long long m = xm ? P.xmasks[(size_t)k * GMAX] : 0ull;
+            if ((t & 31) == 0) {
+                L.load(P, I, t, lane);
+                aj_n = load_atom<T>(P, __shfl_sync(FULL, L.e.x, 0) * CL + jj, R, K);
+            }
+            const int2 e = make_int2(__shfl_sync(FULL, L.e.x, t & 31), __shfl_sync(FULL, L.e.y, t & 31));
+            const unsigned long long m = __shfl_sync(FULL, L.m, t & 31);
+            Atom<T> aj = aj_n;
+            if (((t + 1) & 31) != 0 && t + 1 < ntot)
+                aj_n = load_atom<T>(P, __shfl_sync(FULL, L.e.x, (t + 1) & 31) * CL + jj, R, K);
             const int jlig = entry_jlig(e.y);
             const LigState<T> S = lig_state<T>(P, R, jlig);
             float sx, sy, sz;
             entry_shift(e.y, R.box[0], R.box[1], R.box[2], sx, sy, sz);
             const int ja = e.x * CL + jj;
-            Atom<T> aj = load_atom<T>(P, ja, R, K);
             aj.x = rel_img<T>((float)aj.x, sx, c.x);
             aj.y = rel_img<T>((float)aj.y, sy, c.y);
             aj.z = rel_img<T>((float)aj.z, sz, c.z);
@@ -625,17 +680,22 @@ __global__ void __launch_bounds__(128) k_lig(DevPtrs P) {
             }
         }
         red_iforce<T>(P, I.c0 * CL, ii, jj, fi0, fi1);
-        if (!ENERGY) continue;
-        const int slot_map[6] = {EA_LIGENV_LJ, EA_LIGLIG_LJ, EA_LIGENV_C, EA_LIGLIG_C, EA_DUDLV,
-                                 EA_DUDLQ};
+        if (ENERGY) {
+            const int slot_map[6] = {EA_LIGENV_LJ, EA_LIGLIG_LJ, EA_LIGENV_C, EA_LIGLIG_C, EA_DUDLV,
+                                     EA_DUDLQ};
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            const double s = warp_sum<double>(acc[q]);
-            if (lane == 0) {
-                if (!isfinite(s)) set_err(P.cnt, ERRB_NONFINITE, I.rep);
-                if (s != 0.0) add_fixed(P.eacc + (size_t)I.rep * EA_N + slot_map[q], to_fixed_d(s));
+            for (int q = 0; q < 6; ++q) {
+                const double s = warp_sum<double>(acc[q]);
+                if (lane == 0) {
+                    if (!isfinite(s)) set_err(P.cnt, ERRB_NONFINITE, I.rep);
+                    if (s != 0.0)
+                        add_fixed(P.eacc + (size_t)I.rep * EA_N + slot_map[q], to_fixed_d(s));
+                }
             }
         }
+        if (nw >= n_items) break;
+        if (lane == 0) it = nw + atomicAdd(&P.cnt->lig_next, 1);
+        it = __shfl_sync(FULL, it, 0);
     }
 }
 
@@ -845,21 +905,34 @@ __global__ void __launch_bounds__(128) k_count_lig(DevPtrs P) {
 
 }  // namespace
 
+// Small systems: at most ENV_SMALL_ITEMS clusters per SM give each scheduler a
+// warp or two, whatever the registers allow: there the kernel is bound by one
+// warp's latency, and the variant with 255 registers interleaves the eight pairs
+// of a row.
+constexpr int ENV_SMALL_ITEMS = 8;
+static bool env_small(const DevPtrs& P, int n_sm) { return P.C <= ENV_SMALL_ITEMS * n_sm; }
+
 void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precision, int grid,
-                       int block) {
-    if (precision == 1) k_env_rows<double, true><<<grid, block, 0, s>>>(P);
-    else if (energy) k_env_rows<float, true><<<grid, block, 0, s>>>(P);
-    else k_env_rows<float, false><<<grid, block, 0, s>>>(P);
+                       int block, int n_sm) {
+    if (precision == 1) {
+        k_env_rows<double, true, 2><<<grid, block, 0, s>>>(P);
+    } else if (env_small(P, n_sm)) {
+        if (energy) k_env_rows<float, true, 1><<<grid, block, 0, s>>>(P);
+        else k_env_rows<float, false, 1><<<grid, block, 0, s>>>(P);
+    } else {
+        if (energy) k_env_rows<float, true, 3><<<grid, block, 0, s>>>(P);
+        else k_env_rows<float, false, 4><<<grid, block, 0, s>>>(P);
+    }
 }
 
 int env_kernel_occupancy(int block, int precision, bool energy) {
     int nb = 0;
     if (precision == 1)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<double, true>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<double, true, 2>, block, 0);
     else if (energy)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, true>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, true, 3>, block, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, false>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, false, 4>, block, 0);
     return nb;
 }
 
