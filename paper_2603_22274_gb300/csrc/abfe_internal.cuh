@@ -181,6 +181,7 @@ struct Counters {
     int n_rebuilds;
     int build_next;                // work counter of the list builder (cluster chunks)
     int prune;                     // 1 = re-prune the inner list in this step
+    int blocks_done;               // blocks of the integrator that have finished
     unsigned int dispb2;           // float bits: max squared displacement of this step's
                                    // positions from the outer build's positions
     unsigned int last_dispb2;      // dispb2 of the last finished step (read by the
@@ -433,11 +434,13 @@ void launch_lig_forces(const DevPtrs& P, cudaStream_t s, int precision, int grid
                        bool energy);
 void launch_lig_ukn(const DevPtrs& P, cudaStream_t s, int grid, int precision);
 void launch_count_pairs(const DevPtrs& P, cudaStream_t s, int grid, int block);
-void launch_integrate(const DevPtrs& P, cudaStream_t s, int n_sm);
-void launch_step_end(const DevPtrs& P, cudaStream_t s, int inc_step, int force_rebuild,
-                     int force_prune, cudaGraphConditionalHandle h_rebuild,
-                     cudaGraphConditionalHandle h_prune, cudaGraphConditionalHandle h_exchange,
-                     int use_handle);
+// what the integrator's last block does after it (on = 0: nothing): count the
+// step, decide on rebuilds and prunes (forced ones too), set the graph conditionals
+struct StepEnd {
+    int on = 0, inc_step = 0, force_rebuild = 0, force_prune = 0, use_handle = 0;
+    cudaGraphConditionalHandle h_update = 0, h_exchange = 0;
+};
+void launch_integrate(const DevPtrs& P, cudaStream_t s, int n_sm, const StepEnd& end = StepEnd{});
 void launch_bonds(const DevPtrs& P, cudaStream_t s, int precision, bool energy);
 // alchemical waters: slot charges at every replica's lambda_q; energy-pass sums
 void launch_aw_refresh(const DevPtrs& P, cudaStream_t s);

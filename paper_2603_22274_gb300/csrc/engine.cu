@@ -16,6 +16,8 @@
 #include <cstdio>
 #include <cstring>
 #include <fstream>
+#include <functional>
+#include <initializer_list>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -347,11 +349,19 @@ void enqueue_forces(abfe_ctx* c, cudaStream_t s, bool energy, bool fork = true) 
     }
 }
 
+// list decisions without a step
+StepEnd forced_end(bool rebuild, bool prune) {
+    StepEnd e;
+    e.on = 1;
+    e.force_rebuild = rebuild ? 1 : 0;
+    e.force_prune = prune ? 1 : 0;
+    return e;
+}
+
 // zero forces, displacement check, rebuild and prune decisions, (predicated)
 // outer rebuild and prune
 void enqueue_prepare(abfe_ctx* c, cudaStream_t s) {
-    launch_integrate(with_sp(c, SP_ZERO), s, c->n_sm);
-    launch_step_end(c->P, s, 0, c->force_rebuild ? 1 : 0, c->force_prune ? 1 : 0, 0, 0, 0, 0);
+    launch_integrate(with_sp(c, SP_ZERO), s, c->n_sm, forced_end(c->force_rebuild, c->force_prune));
     // host-forced builds and prunes are timed while profiling is on
     const bool tb = c->force_rebuild, tp = c->force_rebuild || c->force_prune;
     if (tb) prof_rec(c, c->ev_build, true, s);
@@ -1646,10 +1656,11 @@ static void enqueue_exchange(abfe_ctx* c, cudaStream_t s, bool fork) {
     launch_integrate(with_sp(c, SP_XPRE), s, c->n_sm);
 }
 
-// Appends an IF conditional node to the capture of stream s, with its handle
-// (default 0), and records `body` into the node's graph through the side stream.
-template <class F>
-static bool capture_if(abfe_ctx* c, cudaStream_t s, cudaGraphConditionalHandle h, F body) {
+// Appends a conditional node of `n` bodies (a switch on the handle's value, or an
+// if for a single body) to the capture of stream s and records the bodies into
+// the node's graphs through the side stream.
+static bool capture_cond(abfe_ctx* c, cudaStream_t s, cudaGraphConditionalHandle h,
+                         std::initializer_list<std::function<void(cudaStream_t)>> bodies) {
     cudaStreamCaptureStatus cs;
     unsigned long long id;
     cudaGraph_t g;
@@ -1660,18 +1671,21 @@ static bool capture_if(abfe_ctx* c, cudaStream_t s, cudaGraphConditionalHandle h
     cudaGraphNodeParams np = {};
     np.type = cudaGraphNodeTypeConditional;
     np.conditional.handle = h;
-    np.conditional.type = cudaGraphCondTypeIf;
-    np.conditional.size = 1;
+    np.conditional.type = bodies.size() > 1 ? cudaGraphCondTypeSwitch : cudaGraphCondTypeIf;
+    np.conditional.size = (unsigned int)bodies.size();
     cudaGraphNode_t cn;
     if (cudaGraphAddNode(&cn, g, deps, ed, nd, &np) != cudaSuccess) return false;
-    cudaGraph_t gbody = np.conditional.phGraph_out[0];
-    // the side stream only ever records into the body graph: launch nothing on
-    // it unless its capture began
-    if (cudaStreamBeginCaptureToGraph(c->side, gbody, nullptr, nullptr, 0,
-                                      cudaStreamCaptureModeRelaxed) != cudaSuccess)
-        return false;
-    body(c->side);
-    if (cudaStreamEndCapture(c->side, &gbody) != cudaSuccess) return false;
+    int k = 0;
+    for (const auto& body : bodies) {
+        cudaGraph_t gbody = np.conditional.phGraph_out[k++];
+        // the side stream only ever records into the body graph: launch nothing on
+        // it unless its capture began
+        if (cudaStreamBeginCaptureToGraph(c->side, gbody, nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeRelaxed) != cudaSuccess)
+            return false;
+        body(c->side);
+        if (cudaStreamEndCapture(c->side, &gbody) != cudaSuccess) return false;
+    }
     return cudaStreamUpdateCaptureDependencies(s, &cn, nullptr, 1,
                                                cudaStreamSetCaptureDependencies) == cudaSuccess;
 }
@@ -1679,43 +1693,49 @@ static bool capture_if(abfe_ctx* c, cudaStream_t s, cudaGraphConditionalHandle h
 extern "C" {
 
 static bool enqueue_step(abfe_ctx* c, cudaStream_t s, int mode) {
-    // mode 0: direct launches; 1: capture with conditional rebuild, prune and
-    // exchange nodes; 2: predicated capture
-    cudaGraphConditionalHandle h_ex = 0;
-    prof_rec(c, c->ev_int, true, s);
-    launch_integrate(with_sp(c, SP_STEP), s, c->n_sm);
-    prof_rec(c, c->ev_int, false, s);
+    // mode 0: direct launches; 1: capture with a conditional node for the list
+    // updates and one for the exchange; 2: predicated capture
+    StepEnd end;
+    end.on = 1;
+    end.inc_step = 1;
     if (mode == 1) {
         cudaStreamCaptureStatus cs;
         unsigned long long id;
         cudaGraph_t g;
         if (cudaStreamGetCaptureInfo(s, &cs, &id, &g, nullptr, nullptr, nullptr) != cudaSuccess)
             return false;
-        cudaGraphConditionalHandle h_rb, h_pr;
-        if (cudaGraphConditionalHandleCreate(&h_rb, g, 0, 0) != cudaSuccess) return false;
-        if (cudaGraphConditionalHandleCreate(&h_pr, g, 0, 0) != cudaSuccess) return false;
-        if (c->ex_every > 0 && cudaGraphConditionalHandleCreate(&h_ex, g, 0, 0) != cudaSuccess)
+        end.use_handle = 1;
+        if (cudaGraphConditionalHandleCreate(&end.h_update, g, 2, 0) != cudaSuccess) return false;
+        if (c->ex_every > 0 &&
+            cudaGraphConditionalHandleCreate(&end.h_exchange, g, 0, 0) != cudaSuccess)
             return false;
-        launch_step_end(c->P, s, 1, 0, 0, h_rb, h_pr, h_ex, 1);
-        if (!capture_if(c, s, h_rb, [&](cudaStream_t b) {
-                launch_rebuild(c->P, b, c->n_sm);
-                launch_list_build(c->P, b, c->max_lig_cl);
-            }))
-            return false;
-        if (!capture_if(c, s, h_pr, [&](cudaStream_t b) { launch_prune(c->P, b, c->n_sm); }))
+    } else if (mode == 2 && c->ex_every > 0) {
+        return false;   // the predicated form has no place for an exchange: only direct launches do
+    }
+    prof_rec(c, c->ev_int, true, s);
+    launch_integrate(with_sp(c, SP_STEP), s, c->n_sm, end);
+    prof_rec(c, c->ev_int, false, s);
+    auto rebuild = [&](cudaStream_t b) {
+        launch_rebuild(c->P, b, c->n_sm);
+        launch_list_build(c->P, b, c->max_lig_cl);
+    };
+    auto prune = [&](cudaStream_t b) { launch_prune(c->P, b, c->n_sm); };
+    if (mode == 1) {
+        // one node for both updates: a conditional node costs 6 us whether it is
+        // taken or not, more than the launches that it skips
+        if (!capture_cond(c, s, end.h_update, {prune, [&](cudaStream_t b) {
+                                                   rebuild(b);
+                                                   prune(b);
+                                               }}))
             return false;
     } else {
-        // the predicated form has no place for an exchange: only direct launches do
-        if (mode == 2 && c->ex_every > 0) return false;
-        launch_step_end(c->P, s, 1, 0, 0, 0, 0, 0, 0);
-        launch_rebuild(c->P, s, c->n_sm);
-        launch_list_build(c->P, s, c->max_lig_cl);
-        launch_prune(c->P, s, c->n_sm);
+        rebuild(s);
+        prune(s);
     }
     enqueue_forces(c, s, false);
     if (c->ex_every > 0) {
         if (mode == 1) {
-            if (!capture_if(c, s, h_ex, [&](cudaStream_t b) { enqueue_exchange(c, b, false); }))
+            if (!capture_cond(c, s, end.h_exchange, {[&](cudaStream_t b) { enqueue_exchange(c, b, false); }}))
                 return false;
         } else {
             c->dev_step += 1;
@@ -2258,8 +2278,7 @@ abfe_status abfe_autotune(abfe_ctx* c, const char* cache_path, int32_t reps) {
         prune_ms = env_ms = 0.f;
         for (int i = 0; i <= reps; ++i) {    // the first round warms up
             c->force_prune = true;
-            launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm);
-            launch_step_end(c->P, c->stream, 0, 0, 1, 0, 0, 0, 0);
+            launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm, forced_end(false, true));
             cudaEventRecord(e0, c->stream);
             launch_prune(c->P, c->stream, c->n_sm);
             cudaEventRecord(e1, c->stream);
@@ -2376,8 +2395,7 @@ abfe_status abfe_autotune_cadence(abfe_ctx* c, double dt, double gamma, uint64_t
     CK(cudaEventCreate(&e1));
     CK(cudaEventCreate(&e2));
     auto timed = [&](bool rebuild, float& build_ms, float& prune_ms, float& env_ms) -> bool {
-        launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm);
-        launch_step_end(c->P, c->stream, 0, rebuild ? 1 : 0, 1, 0, 0, 0, 0);
+        launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm, forced_end(rebuild, true));
         cudaEventRecord(e0, c->stream);
         launch_rebuild(c->P, c->stream, c->n_sm);
         launch_list_build(c->P, c->stream, c->max_lig_cl);

@@ -4,9 +4,8 @@
 //   fixed-point force, then (drift) A - O - A of BAOAB (Leimkuhler & Matthews
 //   2013) with Philox4x32-10 normals (Salmon et al., SC'11) by Box-Muller,
 //   clear the force accumulators, and the max squared displacement since the
-//   last prune (drives the prune and rebuild decisions).
-// * k_step_end: step counter, rebuild and prune flags, optional CUDA-graph
-//   conditionals.
+//   last prune; its last block ends the step (step counter, rebuild and prune
+//   flags, CUDA-graph conditionals).
 // * k_bonds: harmonic bonds (keep the synthetic molecules together).
 // * k_restraints: the FP64 bonded terms, a block per replica: the six-term Boresch
 //   restraint (paper, section "Restraints") and the periodic torsions of the
@@ -116,116 +115,42 @@ __global__ void k_exchange_done(Counters* c, const int* n_acc) {
     c->ex_accepted += *n_acc;
 }
 
+// fixed point to float, correctly rounded: the magnitude normalised to 32 bits
+// with its lost bits ORed into the last one, then a 32-bit conversion. (Through
+// double it took three instructions on the FP64 pipe, 207 issue cycles per warp
+// against 46.)
 __device__ __forceinline__ float fixed_to_float(long long v) {
-    return (float)((double)v * INV_FSCALE);
-}
-
-__global__ void __launch_bounds__(256) k_integrate(DevPtrs P) {
-    const StepParams sp = *P.sp;
-    const unsigned long long step = P.cnt->step;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        P.cnt->env_next = 0;
-        P.cnt->lig_next = 0;
-    }
-    // this step's energy sums start from zero
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.R * EA_N; i += gridDim.x * blockDim.x)
-        P.eacc[i] = 0;
-    const int lane = threadIdx.x & 31;
-    const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    float dmax = 0.0f, bmax = 0.0f;
-    bool bad = false;
-    for (int base = warp_global * 32; base < P.S; base += nwarps * 32) {
-        const int s = base + lane;
-        const int o = s < P.S ? P.orig[s] : -1;
-        float d2 = 0.0f;   // squared displacement from the replica's prune positions
-        float b2 = 0.0f;   // and from its outer-build positions
-        if (o >= 0) {
-            float4 x = P.xq[s];
-            float4 v = P.v[s];
-            const float invm = v.w;
-            const float fxs = fixed_to_float(P.fx[s]), fys = fixed_to_float(P.fy[s]),
-                        fzs = fixed_to_float(P.fz[s]);
-            const float kk = sp.kick * invm;
-            v.x = fmaf(kk, fxs, v.x);
-            v.y = fmaf(kk, fys, v.y);
-            v.z = fmaf(kk, fzs, v.z);
-            if (sp.drift) {
-                x.x = fmaf(sp.half_dt, v.x, x.x);
-                x.y = fmaf(sp.half_dt, v.y, x.y);
-                x.z = fmaf(sp.half_dt, v.z, x.z);
-                const int rep = P.rep_of_cl[s >> 3];
-                const float3 z = gauss3((unsigned int)o, step, (unsigned int)rep, sp.seed);
-                const float sd = sp.c2 * sqrtf(invm);
-                v.x = fmaf(sp.c1, v.x, sd * z.x);
-                v.y = fmaf(sp.c1, v.y, sd * z.y);
-                v.z = fmaf(sp.c1, v.z, sd * z.z);
-                x.x = fmaf(sp.half_dt, v.x, x.x);
-                x.y = fmaf(sp.half_dt, v.y, x.y);
-                x.z = fmaf(sp.half_dt, v.z, x.z);
-            }
-            if (sp.zero_force) {
-                P.fx[s] = 0; P.fy[s] = 0; P.fz[s] = 0;
-            }
-            if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
-                  isfinite(v.y) && isfinite(v.z)))
-                bad = true;
-            P.xq[s] = x;
-            P.v[s] = v;
-            const float4 r = P.xref[s], b = P.xbuild[s];
-            const float dx = x.x - r.x, dy = x.y - r.y, dz = x.z - r.z;
-            d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            const float bx = x.x - b.x, by = x.y - b.y, bz = x.z - b.z;
-            b2 = fmaf(bx, bx, fmaf(by, by, bz * bz));
-        }
-        dmax = fmaxf(dmax, d2);
-        bmax = fmaxf(bmax, b2);
-        // per replica: the largest over each cluster (8 lanes, one replica),
-        // added once per warp when its 32 slots share a replica
-        const int rep = s < P.S ? P.rep_of_cl[s >> 3] : -1;
-        const bool one = __all_sync(FULL, rep == __shfl_sync(FULL, rep, 0));
-        float m = d2, mb = b2;
-        for (int k = 1; k < (one ? 32 : 8); k <<= 1) {
-            m = fmaxf(m, __shfl_xor_sync(FULL, m, k));
-            mb = fmaxf(mb, __shfl_xor_sync(FULL, mb, k));
-        }
-        if (rep >= 0 && (lane & (one ? 31 : 7)) == 0) {
-            if (m > 0.0f) atomicMax(&P.disp_r[rep], __float_as_uint(m));
-            if (mb > 0.0f) atomicMax(&P.dispb_r[rep], __float_as_uint(mb));
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        dmax = fmaxf(dmax, __shfl_xor_sync(FULL, dmax, o));
-        bmax = fmaxf(bmax, __shfl_xor_sync(FULL, bmax, o));
-    }
-    if (lane == 0 && dmax > 0.0f) atomicMax(&P.cnt->maxdisp2, __float_as_uint(dmax));
-    if (lane == 0 && bmax > 0.0f) atomicMax(&P.cnt->dispb2, __float_as_uint(bmax));
-    if (bad) set_err(P.cnt, ERRB_NONFINITE, -1);
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int z = __clzll((long long)a);
+    const unsigned long long n = a << (z & 63);
+    const float m = __uint2float_rn((unsigned int)(n >> 32) | ((unsigned int)n != 0u ? 1u : 0u));
+    const float f = a ? m * __int_as_float((127 - z) << 23) : 0.0f;   // m 2^(32 - z) 2^-32
+    return v < 0 ? -f : f;
 }
 
 // Step counter and the list decisions for this step, from the displacements
-// the integrator measured: re-prune the inner list of every replica one of
-// whose atoms now lies more than prune_skin/2 from its position at that
-// replica's last prune; rebuild the outer list when an atom now lies more
-// than skin/2 from its position at the outer build (the list holds every pair
-// within r_c + skin there, so every pair within r_c now); a rebuild is always
-// followed by a prune; both per replica (the replicas whose own atoms moved).
-__global__ void __launch_bounds__(256) k_step_end(DevPtrs P, int inc_step, int force_rebuild,
-                                                  int force_prune, cudaGraphConditionalHandle h_rb,
-                                                  cudaGraphConditionalHandle h_pr,
-                                                  cudaGraphConditionalHandle h_ex, int use_handle) {
+// the integrator measured (one block, 256 threads): re-prune the inner list of
+// every replica one of whose atoms now lies more than prune_skin/2 from its
+// position at that replica's last prune; rebuild the outer list when an atom now
+// lies more than skin/2 from its position at the outer build (the list holds
+// every pair within r_c + skin there, so every pair within r_c now); a rebuild is
+// always followed by a prune; both per replica (the replicas whose own atoms
+// moved).
+__device__ __forceinline__ void step_end(const DevPtrs& P, const StepEnd& E) {
     Counters* c = P.cnt;
     __shared__ int s_rb, s_pr;
     if (threadIdx.x == 0) {
-        if (inc_step) c->step += 1ull;
-        const float d2 = __uint_as_float(c->maxdisp2);
-        const float db2 = __uint_as_float(c->dispb2);
+        const unsigned long long step = c->step + (E.inc_step ? 1ull : 0ull);
+        c->step = step;
+        const unsigned int db = __ldcg(&c->dispb2);
+        const float d2 = __uint_as_float(__ldcg(&c->maxdisp2));
+        const float db2 = __uint_as_float(db);
         const bool nan = !(d2 == d2) || !(db2 == db2);
-        const int rb = (force_rebuild || nan || db2 > P.skin_out_half2) ? 1 : 0;
-        c->last_dispb2 = c->dispb2;
+        const int rb = (E.force_rebuild || nan || db2 > P.skin_out_half2) ? 1 : 0;
+        c->last_dispb2 = db;
         c->dispb2 = 0u;     // both measured afresh by every step's integrator
         c->maxdisp2 = 0u;
-        const int pr = (rb || force_prune || d2 > P.skin_in_half2) ? 1 : 0;
+        const int pr = (rb || E.force_prune || d2 > P.skin_in_half2) ? 1 : 0;
         c->rebuild = rb;
         c->prune = pr;
         if (pr) {
@@ -234,12 +159,12 @@ __global__ void __launch_bounds__(256) k_step_end(DevPtrs P, int inc_step, int f
         }
         s_rb = rb;
         s_pr = pr;
-        if (use_handle) {
-            cudaGraphSetConditional(h_rb, (unsigned int)rb);
-            cudaGraphSetConditional(h_pr, (unsigned int)pr);
+        if (E.use_handle) {
+            // bodies of the update node: 0 prune, 1 rebuild and prune, else nothing
+            cudaGraphSetConditional(E.h_update, rb ? 1u : (pr ? 0u : 2u));
             // a replica-exchange attempt ends every ex_every-th step
             if (P.ex_every > 0)
-                cudaGraphSetConditional(h_ex, (c->step % (unsigned long long)P.ex_every) == 0ull ? 1u : 0u);
+                cudaGraphSetConditional(E.h_exchange, (step % (unsigned long long)P.ex_every) == 0ull ? 1u : 0u);
         }
     }
     __syncthreads();
@@ -253,9 +178,9 @@ __global__ void __launch_bounds__(256) k_step_end(DevPtrs P, int inc_step, int f
     // group into fewer events, each with fixed costs.
     constexpr float JOIN2 = 0.5625f;   // (3/4)^2
     for (int r = threadIdx.x; r < P.R; r += blockDim.x) {
-        const float dr = __uint_as_float(P.disp_r[r]), db = __uint_as_float(P.dispb_r[r]);
-        const int b = s_rb && (force_rebuild || !(db <= JOIN2 * P.skin_out_half2)) ? 1 : 0;
-        const int f = s_pr && (b || force_prune || !(dr <= JOIN2 * P.skin_in_half2)) ? 1 : 0;
+        const float dr = __uint_as_float(__ldcg(&P.disp_r[r])), db = __uint_as_float(__ldcg(&P.dispb_r[r]));
+        const int b = s_rb && (E.force_rebuild || !(db <= JOIN2 * P.skin_out_half2)) ? 1 : 0;
+        const int f = s_pr && (b || E.force_prune || !(dr <= JOIN2 * P.skin_in_half2)) ? 1 : 0;
         P.bflag[r] = b;
         P.pflag[r] = f;
         P.disp_r[r] = 0u;
@@ -282,6 +207,106 @@ __global__ void __launch_bounds__(256) k_step_end(DevPtrs P, int inc_step, int f
         atomicAdd(&c->n_win_rebuilds, (unsigned long long)nb);
         atomicAdd(&c->n_win_prunes, (unsigned long long)np);
     }
+}
+
+// E.on: the last block to finish ends the step (step_end), which saves the
+// launch of its own that a one-block kernel took (3.3 us of a 62 us step of one
+// solvent window).
+__global__ void __launch_bounds__(256) k_integrate(DevPtrs P, StepEnd E) {
+    const StepParams sp = *P.sp;
+    const unsigned long long step = P.cnt->step;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        P.cnt->env_next = 0;
+        P.cnt->lig_next = 0;
+    }
+    // this step's energy sums start from zero
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.R * EA_N; i += gridDim.x * blockDim.x)
+        P.eacc[i] = 0;
+    const int lane = threadIdx.x & 31;
+    const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    // one slot per thread (small systems): load everything at once, without
+    // waiting for the original index to tell the padding slots
+    const bool eager = nwarps * 32 >= P.S;
+    float dmax = 0.0f, bmax = 0.0f;
+    bool bad = false;
+    for (int base = warp_global * 32; base < P.S; base += nwarps * 32) {
+        const int s = base + lane;
+        const int o = s < P.S ? P.orig[s] : -1;
+        const int rep = s < P.S ? P.rep_of_cl[s >> 3] : -1;
+        float d2 = 0.0f;   // squared displacement from the replica's prune positions
+        float b2 = 0.0f;   // and from its outer-build positions
+        if ((eager && s < P.S) || o >= 0) {
+            float4 x = P.xq[s];
+            float4 v = P.v[s];
+            const long long fx = P.fx[s], fy = P.fy[s], fz = P.fz[s];
+            const float4 r = P.xref[s], b = P.xbuild[s];
+            const float invm = v.w;
+            const float fxs = fixed_to_float(fx), fys = fixed_to_float(fy), fzs = fixed_to_float(fz);
+            const float kk = sp.kick * invm;
+            v.x = fmaf(kk, fxs, v.x);
+            v.y = fmaf(kk, fys, v.y);
+            v.z = fmaf(kk, fzs, v.z);
+            if (sp.drift) {
+                x.x = fmaf(sp.half_dt, v.x, x.x);
+                x.y = fmaf(sp.half_dt, v.y, x.y);
+                x.z = fmaf(sp.half_dt, v.z, x.z);
+                const float3 z = gauss3((unsigned int)o, step, (unsigned int)rep, sp.seed);
+                const float sd = sp.c2 * sqrtf(invm);
+                v.x = fmaf(sp.c1, v.x, sd * z.x);
+                v.y = fmaf(sp.c1, v.y, sd * z.y);
+                v.z = fmaf(sp.c1, v.z, sd * z.z);
+                x.x = fmaf(sp.half_dt, v.x, x.x);
+                x.y = fmaf(sp.half_dt, v.y, x.y);
+                x.z = fmaf(sp.half_dt, v.z, x.z);
+            }
+            if (o >= 0) {
+                if (sp.zero_force) {
+                    P.fx[s] = 0; P.fy[s] = 0; P.fz[s] = 0;
+                }
+                if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
+                      isfinite(v.y) && isfinite(v.z)))
+                    bad = true;
+                P.xq[s] = x;
+                P.v[s] = v;
+                const float dx = x.x - r.x, dy = x.y - r.y, dz = x.z - r.z;
+                d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                const float bx = x.x - b.x, by = x.y - b.y, bz = x.z - b.z;
+                b2 = fmaf(bx, bx, fmaf(by, by, bz * bz));
+            }
+        }
+        dmax = fmaxf(dmax, d2);
+        bmax = fmaxf(bmax, b2);
+        // per replica: the largest over each cluster (8 lanes, one replica),
+        // added once per warp when its 32 slots share a replica
+        const bool one = __all_sync(FULL, rep == __shfl_sync(FULL, rep, 0));
+        float m = d2, mb = b2;
+        for (int k = 1; k < (one ? 32 : 8); k <<= 1) {
+            m = fmaxf(m, __shfl_xor_sync(FULL, m, k));
+            mb = fmaxf(mb, __shfl_xor_sync(FULL, mb, k));
+        }
+        if (rep >= 0 && (lane & (one ? 31 : 7)) == 0) {
+            if (m > 0.0f) atomicMax(&P.disp_r[rep], __float_as_uint(m));
+            if (mb > 0.0f) atomicMax(&P.dispb_r[rep], __float_as_uint(mb));
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        dmax = fmaxf(dmax, __shfl_xor_sync(FULL, dmax, o));
+        bmax = fmaxf(bmax, __shfl_xor_sync(FULL, bmax, o));
+    }
+    if (lane == 0 && dmax > 0.0f) atomicMax(&P.cnt->maxdisp2, __float_as_uint(dmax));
+    if (lane == 0 && bmax > 0.0f) atomicMax(&P.cnt->dispb2, __float_as_uint(bmax));
+    if (bad) set_err(P.cnt, ERRB_NONFINITE, -1);
+    if (!E.on) return;
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&P.cnt->blocks_done, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) P.cnt->blocks_done = 0;
+    step_end(P, E);
 }
 
 template <typename T>
@@ -816,18 +841,10 @@ __global__ void k_gather_in(DevPtrs P, int what, const double* in) {
 
 }  // namespace
 
-void launch_integrate(const DevPtrs& P, cudaStream_t s, int n_sm) {
+void launch_integrate(const DevPtrs& P, cudaStream_t s, int n_sm, const StepEnd& end) {
     const int tb = 256;
     const int grid = max(1, min((P.S + tb - 1) / tb, n_sm * 8));
-    k_integrate<<<grid, tb, 0, s>>>(P);
-}
-
-void launch_step_end(const DevPtrs& P, cudaStream_t s, int inc_step, int force_rebuild,
-                     int force_prune, cudaGraphConditionalHandle h_rebuild,
-                     cudaGraphConditionalHandle h_prune, cudaGraphConditionalHandle h_exchange,
-                     int use_handle) {
-    k_step_end<<<1, 256, 0, s>>>(P, inc_step, force_rebuild, force_prune, h_rebuild, h_prune,
-                               h_exchange, use_handle);
+    k_integrate<<<grid, tb, 0, s>>>(P, end);
 }
 
 void launch_bonds(const DevPtrs& P, cudaStream_t s, int precision, bool energy) {
