@@ -385,9 +385,8 @@ abfe_status abfe_load_checkpoint(abfe_ctx *ctx, const char *path);
  *  - Device data are not validated on the host: a lig_idx entry outside
  *    [0, n_atoms) is never dereferenced; it turns every du[k] of that call
  *    into NaN. Anchor indices (host values) are checked.
- *  - Cost: every ligand atom scans all n_atoms atoms once per 16 states
- *    (ceil(K / 16) passes); one call is n_lig x ceil(K / 16) x n_atoms pair
- *    tests in FP64.
+ *  - Cost: one launch; n_lig x n_atoms pair tests in FP32, and for the pairs that
+ *    pass them an exact FP64 test and one FP64 division per distinct lambda_v.
  */
 #define ABFE_NOALLOC_MAX_ATOMS (1 << 22)
 #define ABFE_NOALLOC_MAX_LIG 1024
