@@ -29,6 +29,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "abfe_internal.cuh"
 
@@ -909,7 +910,7 @@ __device__ __forceinline__ float dist2(const float4& a, float x, float y, float 
     return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
-// One warp per outer environment work item, in two passes over its entries.
+// One warp per outer environment work item.
 // (a) Lane per entry: with the clusters' bounding boxes at the current
 // positions, each (entry, i-cluster) is sorted as "no row" (boxes farther
 // apart than the inner radius), "every j atom a row" (farthest points within
@@ -919,12 +920,12 @@ __device__ __forceinline__ float dist2(const float4& a, float x, float y, float 
 // and tests it against all 8 i atoms without branches, in coordinates relative
 // to the i-cluster's box centre: r^2 - r_in^2 = |x_j|^2 + (|x_i|^2 - r_in^2 -
 // 2 x_j.x_i), three FMAs and a min per i atom; a row is live in a half (i
-// atoms 0-3 or 4-7) if the half tile is live and the smallest bracket over
-// the half's atoms that are not excluded is below -|x_j|^2. Rows without
-// excluded pairs go to the plain row list (full rows, then rows with only
-// atoms 0-3, then only atoms 4-7, in range), rows with excluded pairs (masked
-// entries only) to the masked row list with their 8-bit mask of excluded i
-// atoms. Row order within each run follows the outer entries.
+// atoms 0-3 or 4-7) if the smallest bracket over the half's atoms that are not
+// excluded is below -|x_j|^2. (c) Per i-cluster the rows are counted and
+// written, four live entries per pass, in the runs that RowItem describes; rows
+// with excluded pairs (masked entries only) go to the masked row list with
+// their 8-bit mask of excluded i atoms. Row order within each run follows the
+// outer entries.
 // per-warp prune state (dynamic shared memory)
 template <int G>
 struct PrS {
@@ -935,9 +936,8 @@ struct PrS {
     unsigned short test[(PR_ECAP + PR_XCAP) * G];  // queued (entry, i-cluster) tests
     // per (entry, i-cluster): bit jj = row jj has an atom of i atoms 0-3 (lo)
     // or of i atoms 4-7 (hi) inside the inner radius
-    unsigned char lo[PR_ECAP + PR_XCAP][G];
-    unsigned char hi[PR_ECAP + PR_XCAP][G];
-    int ntest;
+    // (bits 0-7 and 8-15)
+    unsigned short lh[PR_ECAP + PR_XCAP][G];
 };
 
 template <int G>
@@ -990,7 +990,6 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_prune(DevPtrs P) {
             S.sh[lane] = make_float4((float)(lane % 3 - 1) * R.box[0],
                                      (float)((lane / 3) % 3 - 1) * R.box[1],
                                      (float)(lane / 9 - 1) * R.box[2], 0.f);
-        if (lane == 0) S.ntest = 0;
         __syncwarp();
         if (lane < G * CL) {
             const int g = lane >> 3;
@@ -1008,17 +1007,19 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_prune(DevPtrs P) {
         }
         __syncwarp();
         const int n_e = I.e_cnt + I.x_cnt;
-        // (a) box classification, lane per entry
-        for (int t0 = 0; t0 < n_e; t0 += 32) {
+        // (a) box classification, lane per entry: the plain entries, then the masked
+        // ones (in batches of their own, so that tests [0, n_tp) need no masks)
+        int n_t = 0, n_tp = 0;
+        for (int t0 = 0; t0 < n_e; t0 = (t0 < I.e_cnt && t0 + 32 > I.e_cnt) ? I.e_cnt : t0 + 32) {
             const int t = t0 + lane;
+            const bool xm = t0 >= I.e_cnt;   // warp-uniform
+            if (xm && t0 == I.e_cnt) n_tp = n_t;
             unsigned int need = 0u;   // bit g: test rows of i-cluster g
-            if (t < n_e) {
-                const bool xm = t >= I.e_cnt;
+            if (t < (xm ? n_e : I.e_cnt)) {
                 const int k = xm ? I.x_begin + (t - I.e_cnt) : I.e_begin + t;
                 const int2 e = xm ? P.xentries[k] : P.entries[k];
-                float sx, sy, sz;
-                entry_shift(e.y, R.box[0], R.box[1], R.box[2], sx, sy, sz);
                 const int code = ((e.y >> 8) & 3) + 3 * ((e.y >> 10) & 3) + 9 * ((e.y >> 12) & 3);
+                const float4 s = S.sh[code];
                 S.word[t] = ((unsigned int)code << ROW_SLOT_BITS) | (unsigned int)(e.x * CL);
                 const float4 jb = P.bbc[e.x], jh = P.bbh[e.x];
                 const unsigned int all = jb.w > 0.f ? (1u << (int)jh.w) - 1u : 0u;
@@ -1027,13 +1028,13 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_prune(DevPtrs P) {
                     unsigned int live = 0u;
                     const float4 ic = S.bb[g][0], ih = S.bb[g][1];
                     if (g < I.ng && entry_g(e.y, g) && all && ic.w > 0.f) {
-                        const float ax = fabsf(jb.x + sx - ic.x), ay = fabsf(jb.y + sy - ic.y),
-                                    az = fabsf(jb.z + sz - ic.z);
-                        const float nx = fmaxf(ax - jh.x - ih.x, 0.f), ny = fmaxf(ay - jh.y - ih.y, 0.f),
-                                    nz = fmaxf(az - jh.z - ih.z, 0.f);
+                        const float ax = fabsf(jb.x + s.x - ic.x), ay = fabsf(jb.y + s.y - ic.y),
+                                    az = fabsf(jb.z + s.z - ic.z);
+                        const float hx = jh.x + ih.x, hy = jh.y + ih.y, hz = jh.z + ih.z;
+                        const float nx = fmaxf(ax - hx, 0.f), ny = fmaxf(ay - hy, 0.f),
+                                    nz = fmaxf(az - hz, 0.f);
                         if (fmaf(nx, nx, fmaf(ny, ny, nz * nz)) < rin2) {
-                            const float fx = ax + jh.x + ih.x, fy = ay + jh.y + ih.y,
-                                        fz = az + jh.z + ih.z;
+                            const float fx = ax + hx, fy = ay + hy, fz = az + hz;
                             const bool masked = xm && P.xmasks[(size_t)k * GMAX + g] != 0ull;
                             if (((e.y >> (2 * g)) & 3) == 3 && !masked &&
                                 fmaf(fx, fx, fmaf(fy, fy, fz * fz)) < rin2)
@@ -1042,8 +1043,7 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_prune(DevPtrs P) {
                                 need |= 1u << g;
                         }
                     }
-                    S.lo[t][g] = (unsigned char)live;
-                    S.hi[t][g] = (unsigned char)live;
+                    S.lh[t][g] = (unsigned short)(live * 0x101u);
                 }
             }
             // queue the tests (order: entry, then i-cluster)
@@ -1051,203 +1051,201 @@ __global__ void __launch_bounds__(PR_WARPS * 32) k_prune(DevPtrs P) {
             for (int g = 0; g < G; ++g) {
                 const bool q = (need >> g) & 1u;
                 const unsigned int b = __ballot_sync(0xffffffffu, q);
-                const int base = S.ntest;
-                if (q) S.test[base + __popc(b & ((1u << lane) - 1u))] = (unsigned short)(t | (g << 10));
-                __syncwarp();
-                if (lane == 0) S.ntest = base + __popc(b);
-                __syncwarp();
+                if (q) S.test[n_t + __popc(b & ((1u << lane) - 1u))] = (unsigned short)(t | (g << 10));
+                n_t += __popc(b);
             }
         }
-        // (b) atom tests, lane per j row, four tests per pass
-        const int n_t = S.ntest;
+        if (I.x_cnt == 0) n_tp = n_t;
+        __syncwarp();
+        // (b) atom tests, lane per j row, NU times four tests per pass (the i atoms read
+        // once for all of them)
         const int jj = lane & 7, sub = lane >> 3;
-        for (int u0 = 0; u0 < n_t; u0 += 4) {
-            const int u = u0 + sub;
-            bool in_lo = false, in_hi = false;
-            int t = 0, g = 0;
-            if (u < n_t) {
-                const int code = S.test[u];
-                t = code & 1023;
-                g = code >> 10;
-                const bool xm = t >= I.e_cnt;
-                const unsigned int wd = S.word[t];
+        auto test_pass = [&](int u0, auto masked, auto nu) {
+            constexpr int NU = decltype(nu)::value;
+            float jx[NU], jy[NU], jz[NU], njn[NU], dm[NU][2];
+            unsigned int ex[NU];
+            int tt[NU], gg[NU];
+            bool on[NU];
+#pragma unroll
+            for (int q = 0; q < NU; ++q) {
+                const int u = u0 + 4 * q + sub;
+                on[q] = u < n_t;
+                const int code = on[q] ? S.test[u] : S.test[u0];
+                tt[q] = code & 1023;
+                gg[q] = G > 1 ? code >> 10 : 0;
+                const unsigned int wd = S.word[tt[q]];
                 const float4 s = S.sh[wd >> ROW_SLOT_BITS];
                 const float4 xj = P.xq[(wd & ROW_SLOT_MASK) + jj];
-                const float4 c = S.bb[g][0];
-                const float jx = xj.x + s.x - c.x, jy = xj.y + s.y - c.y, jz = xj.z + s.z - c.z;
+                const float4 c = S.bb[gg[q]][0];
+                jx[q] = xj.x + s.x - c.x;
+                jy[q] = xj.y + s.y - c.y;
+                jz[q] = xj.z + s.z - c.z;
                 // r^2 - r_in^2 = |x_j|^2 + (|x_i|^2 - r_in^2 - 2 x_i.x_j): the smallest of
                 // the bracket over each half against -|x_j|^2
-                const float njn = -fmaf(jx, jx, fmaf(jy, jy, jz * jz));
-                unsigned int ex = 0u;
-                if (xm) {
+                njn[q] = -fmaf(jx[q], jx[q], fmaf(jy[q], jy[q], jz[q] * jz[q]));
+                ex[q] = 0u;
+                if (masked && tt[q] >= I.e_cnt) {
                     // excluded i atoms of this row: bits jj, jj + 8, ..., jj + 56 of the mask
-                    const int k = I.x_begin + (t - I.e_cnt);
-                    const unsigned long long m = P.xmasks[(size_t)k * GMAX + g];
+                    const int k = I.x_begin + (tt[q] - I.e_cnt);
+                    const unsigned long long m = P.xmasks[(size_t)k * GMAX + gg[q]] >> jj;
 #pragma unroll
-                    for (int ii = 0; ii < CL; ++ii) ex |= (unsigned int)((m >> (ii * 8 + jj)) & 1ull) << ii;
+                    for (int ii = 0; ii < CL; ++ii)
+                        ex[q] |= (unsigned int)((m >> (ii * 8)) & 1ull) << ii;
                 }
-                float dm[2] = {3.0e38f, 3.0e38f};
+                dm[q][0] = dm[q][1] = 3.0e38f;
+            }
 #pragma unroll
-                for (int ii = 0; ii < CL; ++ii) {
-                    const float4 a = S.xi[g * CL + ii];
-                    const float d = fmaf(a.x, jx, fmaf(a.y, jy, fmaf(a.z, jz, a.w)));
-                    dm[ii >> 2] = fminf(dm[ii >> 2], ((ex >> ii) & 1u) ? 3.0e38f : d);
+            for (int ii = 0; ii < CL; ++ii) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (G == 1) a = S.xi[ii];
+#pragma unroll
+                for (int q = 0; q < NU; ++q) {
+                    if (G > 1) a = S.xi[gg[q] * CL + ii];
+                    const float d = fmaf(a.x, jx[q], fmaf(a.y, jy[q], fmaf(a.z, jz[q], a.w)));
+                    dm[q][ii >> 2] =
+                        fminf(dm[q][ii >> 2], masked && ((ex[q] >> ii) & 1u) ? 3.0e38f : d);
                 }
-                // a queued (entry, i-cluster) has both half tiles live: the outer
-                // list is cluster-level
-                in_lo = dm[0] < njn;
-                in_hi = dm[1] < njn;
             }
-            const unsigned int bl = __ballot_sync(0xffffffffu, in_lo);
-            const unsigned int bh = __ballot_sync(0xffffffffu, in_hi);
-            if (u < n_t && jj == 0) {
-                S.lo[t][g] = (unsigned char)((bl >> (8 * sub)) & 0xFFu);
-                S.hi[t][g] = (unsigned char)((bh >> (8 * sub)) & 0xFFu);
+#pragma unroll
+            for (int q = 0; q < NU; ++q) {
+                // a queued (entry, i-cluster) has both half tiles live: the outer list is
+                // cluster-level
+                const unsigned int bl = __ballot_sync(0xffffffffu, dm[q][0] < njn[q]);
+                const unsigned int bh = __ballot_sync(0xffffffffu, dm[q][1] < njn[q]);
+                if (on[q] && jj == 0)
+                    S.lh[tt[q]][gg[q]] = (unsigned short)(((bl >> (8 * sub)) & 0xFFu) |
+                                                          (((bh >> (8 * sub)) & 0xFFu) << 8));
             }
-        }
+        };
+        int u0 = 0;
+        constexpr std::integral_constant<int, 2> TWO{};
+        constexpr std::integral_constant<int, 1> ONE{};
+        for (; u0 + 8 <= n_tp; u0 += 8) test_pass(u0, std::false_type{}, TWO);
+        for (; u0 + 4 <= n_tp; u0 += 4) test_pass(u0, std::false_type{}, ONE);
+        for (; u0 < n_t; u0 += 4) test_pass(u0, std::true_type{}, ONE);
         __syncwarp();
-        // pass 2: row counts per i-cluster: plain rows with both halves in
-        // range (full), with only atoms 0-3 (lo) or only atoms 4-7 (hi), and
-        // masked rows
-        int cf[G], cl[G], ch[G], cx[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) { cf[g] = 0; cl[g] = 0; ch[g] = 0; cx[g] = 0; }
-        for (int t = lane; t < n_e; t += 32) {
-            const bool xm = t >= I.e_cnt;
-            const int k = xm ? I.x_begin + (t - I.e_cnt) : I.e_begin + t;
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                const unsigned int lo = S.lo[t][g], hi = S.hi[t][g];
-                unsigned int exr = 0u;
-                if (xm) {
-                    unsigned long long m = P.xmasks[(size_t)k * GMAX + g];
-                    m |= m >> 32; m |= m >> 16; m |= m >> 8;
-                    exr = (unsigned int)(m & 0xFFull);
+        // (c) per i-cluster: row counts - both halves in range (full), only atoms
+        // 0-3 (lo) or only atoms 4-7 (hi), and masked rows - then the rows
+#pragma unroll 1
+        for (int g = 0; g < I.ng; ++g) {
+            int n_live = 0, n_lp = 0;          // entries with rows, compacted over S.test; plain ones
+            int cf = 0, cl = 0, ch = 0, cx = 0;
+            for (int t0 = 0; t0 < n_e; t0 += 32) {
+                const int t = t0 + lane;
+                unsigned int lo = 0u, hi = 0u;
+                if (t < n_e) {
+                    lo = S.lh[t][g] & 0xFFu;
+                    hi = S.lh[t][g] >> 8;
+                    unsigned int exr = 0u;
+                    if (t >= I.e_cnt) {
+                        unsigned long long m = P.xmasks[(size_t)(I.x_begin + (t - I.e_cnt)) * GMAX + g];
+                        m |= m >> 32; m |= m >> 16; m |= m >> 8;
+                        exr = (unsigned int)(m & 0xFFull);
+                    }
+                    cf += __popc(lo & hi & ~exr);
+                    cl += __popc(lo & ~hi & ~exr);
+                    ch += __popc(hi & ~lo & ~exr);
+                    cx += __popc((lo | hi) & exr);
                 }
-                cf[g] += __popc(lo & hi & ~exr);
-                cl[g] += __popc(lo & ~hi & ~exr);
-                ch[g] += __popc(hi & ~lo & ~exr);
-                cx[g] += __popc((lo | hi) & exr);
+                const bool live = (lo | hi) != 0u;
+                const unsigned int b = __ballot_sync(0xffffffffu, live);
+                if (live) S.test[n_live + __popc(b & ((1u << lane) - 1u))] = (unsigned short)t;
+                n_live += __popc(b);
+                n_lp += __popc(__ballot_sync(0xffffffffu, live && t < I.e_cnt));
             }
-        }
-        int totp = 0, totx = 0, nit = 0;
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            for (int o = 16; o > 0; o >>= 1) {
-                cf[g] += __shfl_xor_sync(0xffffffffu, cf[g], o);
-                cl[g] += __shfl_xor_sync(0xffffffffu, cl[g], o);
-                ch[g] += __shfl_xor_sync(0xffffffffu, ch[g], o);
-                cx[g] += __shfl_xor_sync(0xffffffffu, cx[g], o);
-            }
-            totp += cf[g] + cl[g] + ch[g];
-            totx += cx[g];
-            nit += (cf[g] + cl[g] + ch[g] + cx[g]) > 0 ? 1 : 0;
-        }
-        if (nit == 0) continue;
-        // offsets in this replica's regions
-        unsigned int rb = 0u;
-        int xb = 0, ib = 0;
-        if (lane == 0) {
-            rb = atomicAdd(&P.n_rows_r[I.rep], (unsigned int)totp);
-            xb = atomicAdd(&P.n_xrows_r[I.rep], totx);
-            ib = atomicAdd(&P.n_ritems_r[I.rep], nit);
-        }
-        rb = __shfl_sync(0xffffffffu, rb, 0);
-        xb = __shfl_sync(0xffffffffu, xb, 0);
-        ib = __shfl_sync(0xffffffffu, ib, 0);
-        if ((long long)rb + totp > (long long)P.row_cap[I.rep] ||
-            (long long)xb + totx > P.xrow_cap[I.rep] || (long long)ib + nit > P.ritem_cap[I.rep]) {
+            // (two counts of at most 8 * 576 < 2^16 in one word)
+            const unsigned int s0 = __reduce_add_sync(0xffffffffu, (unsigned int)(cf | (cl << 16)));
+            const unsigned int s1 = __reduce_add_sync(0xffffffffu, (unsigned int)(ch | (cx << 16)));
+            cf = (int)(s0 & 0xFFFFu);
+            cl = (int)(s0 >> 16);
+            ch = (int)(s1 & 0xFFFFu);
+            cx = (int)(s1 >> 16);
+            if (n_live == 0) continue;
+            const int n_row = cf + cl + ch;
+            // offsets in this replica's regions
+            unsigned int rb = 0u;
+            int xb = 0, ib = 0;
             if (lane == 0) {
-                const int k = (long long)rb + totp > (long long)P.row_cap[I.rep] ? OVF_ROWS
-                              : (long long)xb + totx > P.xrow_cap[I.rep]        ? OVF_XROWS
-                                                                                : OVF_RITEMS;
-                const long long need = k == OVF_ROWS ? (long long)rb + totp
-                                       : k == OVF_XROWS ? (long long)xb + totx : (long long)ib + nit;
-                set_err(P.cnt, ERRB_LIST, I.c0, (I.rep << 4) | k, (int)min(need, 2147483647LL));
+                rb = atomicAdd(&P.n_rows_r[I.rep], (unsigned int)n_row);
+                xb = atomicAdd(&P.n_xrows_r[I.rep], cx);
+                ib = atomicAdd(&P.n_ritems_r[I.rep], 1);
             }
-            continue;
-        }
-        rb += P.row_base[I.rep];
-        xb += P.xrow_base[I.rep];
-        ib += P.ritem_base[I.rep];
-        // pass 3: write the rows (lane per entry, warp scans for the offsets) and
-        // items. Per i-cluster: full rows, then rows with only atoms 0-3 in
-        // range (lo), then rows with only atoms 4-7 (hi), each run in entry order.
-        unsigned int ro = rb;
-        int xo = xb, io = ib;
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int nrow = cf[g] + cl[g] + ch[g];
-            if (nrow + cx[g] == 0) continue;
+            rb = __shfl_sync(0xffffffffu, rb, 0);
+            xb = __shfl_sync(0xffffffffu, xb, 0);
+            ib = __shfl_sync(0xffffffffu, ib, 0);
+            if ((long long)rb + n_row > (long long)P.row_cap[I.rep] ||
+                (long long)xb + cx > P.xrow_cap[I.rep] || ib + 1 > P.ritem_cap[I.rep]) {
+                if (lane == 0) {
+                    const int k = (long long)rb + n_row > (long long)P.row_cap[I.rep] ? OVF_ROWS
+                                  : (long long)xb + cx > P.xrow_cap[I.rep]           ? OVF_XROWS
+                                                                                     : OVF_RITEMS;
+                    const long long need = k == OVF_ROWS    ? (long long)rb + n_row
+                                           : k == OVF_XROWS ? (long long)xb + cx
+                                                            : (long long)ib + 1;
+                    set_err(P.cnt, ERRB_LIST, I.c0, (I.rep << 4) | k, (int)min(need, 2147483647LL));
+                }
+                break;
+            }
+            rb += P.row_base[I.rep];
+            xb += P.xrow_base[I.rep];
             if (lane == 0) {
                 RowItem ri;
                 ri.c = I.c0 + g;
-                ri.r_begin = ro;
-                ri.x_begin = xo;
-                ri.cnt = cf[g] | (cx[g] << 16);
-                ri.n_lo = cl[g];
-                ri.n_hi = ch[g];
+                ri.r_begin = rb;
+                ri.x_begin = xb;
+                ri.cnt = cf | (cx << 16);
+                ri.n_lo = cl;
+                ri.n_hi = ch;
                 ri.pad0 = 0;
                 ri.pad1 = 0;
-                P.ritems[io] = ri;
+                P.ritems[ib + P.ritem_base[I.rep]] = ri;
             }
-            ++io;
-            const unsigned int lo_base = ro + (unsigned int)cf[g];
-            const unsigned int hi_base = lo_base + (unsigned int)cl[g];
-            int carf = 0, carl = 0, carh = 0, carx = 0;
-            for (int t0 = 0; t0 < n_e; t0 += 32) {
-                const int t = t0 + lane;
-                unsigned int lo = 0u, hi = 0u, exr = 0u, base = 0u;
-                unsigned long long m = 0ull;
-                if (t < n_e) {
-                    base = S.word[t];
-                    lo = S.lo[t][g];
-                    hi = S.hi[t][g];
-                    if (t >= I.e_cnt) {
-                        m = P.xmasks[(size_t)(I.x_begin + (t - I.e_cnt)) * GMAX + g];
-                        unsigned long long f = m;
-                        f |= f >> 32; f |= f >> 16; f |= f >> 8;
-                        exr = (unsigned int)(f & 0xFFull);
-                    }
-                }
-                const unsigned int mf = lo & hi & ~exr, ml = lo & ~hi & ~exr,
-                                   mh = hi & ~lo & ~exr, mx = (lo | hi) & exr;
-                const int nf = __popc(mf), nl = __popc(ml), nh = __popc(mh), nx = __popc(mx);
-                int sf = nf, sl = nl, shh = nh, sx2 = nx;
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int a0 = __shfl_up_sync(0xffffffffu, sf, o);
-                    const int a1 = __shfl_up_sync(0xffffffffu, sl, o);
-                    const int a2 = __shfl_up_sync(0xffffffffu, shh, o);
-                    const int a3 = __shfl_up_sync(0xffffffffu, sx2, o);
-                    if (lane >= o) { sf += a0; sl += a1; shh += a2; sx2 += a3; }
-                }
-                unsigned int of = ro + (unsigned int)(carf + sf - nf);
-                unsigned int ol = lo_base + (unsigned int)(carl + sl - nl);
-                unsigned int oh = hi_base + (unsigned int)(carh + shh - nh);
-                int ox = xo + carx + sx2 - nx;
-                for (int r = 0; r < CL; ++r) {
-                    const unsigned int word = base + (unsigned int)r;
-                    if ((mf >> r) & 1u) {
-                        P.rows[of++] = word;
-                    } else if ((ml >> r) & 1u) {
-                        P.rows[ol++] = word;
-                    } else if ((mh >> r) & 1u) {
-                        P.rows[oh++] = word;
-                    } else if ((mx >> r) & 1u) {
-                        unsigned int em = 0u;
+            __syncwarp();
+            // lane per row, four live entries per pass: each row takes the next
+            // place of its run (ballot ranks), so a pass writes short contiguous runs
+            unsigned int* full = P.rows + rb;
+            unsigned int* low = full + cf;
+            unsigned int* high = low + cl;
+            int px = 0;
+            const unsigned int lt = (1u << lane) - 1u;
+            for (int v0 = 0; v0 < n_live; v0 += 4) {
+                const bool on = v0 + sub < n_live;
+                const int t = on ? S.test[v0 + sub] : 0;
+                const unsigned int lh = on ? (unsigned int)S.lh[t][g] >> jj : 0u;
+                bool l = lh & 1u, h = lh & 0x100u;
+                const unsigned int word = S.word[t] + (unsigned int)jj;
+                if (v0 + 4 > n_lp) {   // masked entries in this pass (warp-uniform)
+                    unsigned int em = 0u;
+                    if (on && t >= I.e_cnt && (l || h)) {
+                        const unsigned long long m =
+                            P.xmasks[(size_t)(I.x_begin + (t - I.e_cnt)) * GMAX + g] >> jj;
 #pragma unroll
-                        for (int ii = 0; ii < CL; ++ii)
-                            em |= (unsigned int)((m >> (ii * 8 + r)) & 1ull) << ii;
-                        P.xrows[ox++] = make_int2((int)word, (int)em);
+                        for (int ii = 0; ii < CL; ++ii) em |= (unsigned int)((m >> (ii * 8)) & 1ull) << ii;
                     }
+                    const unsigned int bx = __ballot_sync(0xffffffffu, em != 0u);
+                    if (em) {
+                        P.xrows[xb + px + __popc(bx & lt)] = make_int2((int)word, (int)em);
+                        l = h = false;
+                    }
+                    px += __popc(bx);
                 }
-                carf += __shfl_sync(0xffffffffu, sf, 31);
-                carl += __shfl_sync(0xffffffffu, sl, 31);
-                carh += __shfl_sync(0xffffffffu, shh, 31);
-                carx += __shfl_sync(0xffffffffu, sx2, 31);
+                const unsigned int bl = __ballot_sync(0xffffffffu, l);
+                const unsigned int bh = __ballot_sync(0xffffffffu, h);
+                if (bl == bh) {   // full rows only (warp-uniform)
+                    if (l) full[__popc(bl & lt)] = word;
+                    full += __popc(bl);
+                    continue;
+                }
+                const unsigned int mf = bl & bh, ml = bl & ~bh, mh = bh & ~bl;
+                if (l || h) {
+                    const unsigned int m = l ? (h ? mf : ml) : mh;
+                    (l ? (h ? full : low) : high)[__popc(m & lt)] = word;
+                }
+                full += __popc(mf);
+                low += __popc(ml);
+                high += __popc(mh);
             }
-            ro += (unsigned int)nrow;
-            xo += cx[g];
+            __syncwarp();
         }
     }
 }
