@@ -425,7 +425,8 @@ __device__ __forceinline__ int block_prefix(const int* cnt, const int* cap, int*
 // ---------------------------------------------------------------- launch wrappers
 // (defined in the .cu files; all enqueue on the given stream)
 void launch_rebuild(const DevPtrs& P, cudaStream_t s, int n_sm);
-void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl);
+void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl, cudaStream_t s2 = nullptr,
+                       cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
 void launch_prune(const DevPtrs& P, cudaStream_t s, int n_sm);
 void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precision, int grid,
                        int block, int n_sm);

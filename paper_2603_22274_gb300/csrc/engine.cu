@@ -55,7 +55,9 @@ constexpr double PRUNE_SKIN_MAX = 0.15;   // nm: largest inner-list buffer (rows
 struct abfe_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    cudaStream_t side = nullptr;
+    cudaStream_t side = nullptr;           // captures of conditional bodies, and a branch of them
+    cudaStream_t side2 = nullptr;
+    cudaEvent_t ev_side = nullptr, ev_side2 = nullptr;
     cudaStream_t fork = nullptr;           // ligand pair / bond branch
     cudaStream_t fork2 = nullptr;          // restraint / torsion / PME branch
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
@@ -366,7 +368,8 @@ void enqueue_prepare(abfe_ctx* c, cudaStream_t s) {
     const bool tb = c->force_rebuild, tp = c->force_rebuild || c->force_prune;
     if (tb) prof_rec(c, c->ev_build, true, s);
     launch_rebuild(c->P, s, c->n_sm);
-    launch_list_build(c->P, s, c->max_lig_cl);
+    if (tb) launch_list_build(c->P, s, c->max_lig_cl, c->fork, c->ev_fork, c->ev_join);
+    else launch_list_build(c->P, s, c->max_lig_cl);
     if (tb) prof_rec(c, c->ev_build, false, s);
     if (tp) prof_rec(c, c->ev_prune, true, s);
     launch_prune(c->P, s, c->n_sm);
@@ -839,6 +842,9 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         c->own_stream = true;
     }
     cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
+    cudaStreamCreateWithFlags(&c->side2, cudaStreamNonBlocking);
+    cudaEventCreateWithFlags(&c->ev_side, cudaEventDisableTiming);
+    cudaEventCreateWithFlags(&c->ev_side2, cudaEventDisableTiming);
     cudaStreamCreateWithFlags(&c->fork, cudaStreamNonBlocking);
     cudaStreamCreateWithFlags(&c->fork2, cudaStreamNonBlocking);
     cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
@@ -1390,6 +1396,9 @@ void abfe_destroy(abfe_ctx* c) {
     if (!c) return;
     free_all(c);
     if (c->side) cudaStreamDestroy(c->side);
+    if (c->side2) cudaStreamDestroy(c->side2);
+    if (c->ev_side) cudaEventDestroy(c->ev_side);
+    if (c->ev_side2) cudaEventDestroy(c->ev_side2);
     if (c->fork) cudaStreamDestroy(c->fork);
     if (c->fork2) cudaStreamDestroy(c->fork2);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -1717,7 +1726,8 @@ static bool enqueue_step(abfe_ctx* c, cudaStream_t s, int mode) {
     prof_rec(c, c->ev_int, false, s);
     auto rebuild = [&](cudaStream_t b) {
         launch_rebuild(c->P, b, c->n_sm);
-        launch_list_build(c->P, b, c->max_lig_cl);
+        if (mode == 1) launch_list_build(c->P, b, c->max_lig_cl, c->side2, c->ev_side, c->ev_side2);
+        else launch_list_build(c->P, b, c->max_lig_cl);
     };
     auto prune = [&](cudaStream_t b) { launch_prune(c->P, b, c->n_sm); };
     if (mode == 1) {

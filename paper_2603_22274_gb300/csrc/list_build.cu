@@ -159,7 +159,34 @@ __global__ void k_rb_fill(DevPtrs P) {
     }
 }
 
-// One warp per column: bitonic sort of (z bits << 32 | atom index) in shared memory.
+// One warp per column: its atoms in the order of (z bits << 32 | atom index).
+// Columns of at most RANK_MAX atoms by counting, for E atoms per lane, the keys below
+// each: the keys are distinct, so the count is the atom's place. The counts of a lane
+// are independent of each other, where a bitonic sort of 256 keys is 36 dependent
+// passes through shared memory (24 windows of 25,000 atoms 68 -> 29 us; one
+// 60,000-atom complex with columns above 256 atoms 69 -> 21 us).
+constexpr int RANK_MAX = 512;
+template <int E>
+__device__ __forceinline__ void rank_column(const unsigned long long* key, const int* val, int n, int* perm,
+                                            int lane) {
+    unsigned long long mine[E];
+    int rank[E];
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+        mine[q] = lane + 32 * q < n ? key[lane + 32 * q] : 0ull;
+        rank[q] = 0;
+    }
+#pragma unroll 4
+    for (int m = 0; m < n; ++m) {
+        const unsigned long long x = key[m];
+#pragma unroll
+        for (int q = 0; q < E; ++q) rank[q] += x < mine[q] ? 1 : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < E; ++q)
+        if (lane + 32 * q < n) perm[rank[q]] = val[lane + 32 * q];
+}
+
 constexpr int SORT_WARPS = 4;
 __global__ void __launch_bounds__(SORT_WARPS * 32) k_rb_sort(DevPtrs P) {
     if (!P.cnt->rebuild) return;
@@ -175,10 +202,30 @@ __global__ void __launch_bounds__(SORT_WARPS * 32) k_rb_sort(DevPtrs P) {
     const int start = P.col_start[col];
     int n = P.col_fill[col] - start;
     if (n > COL_MAX) n = COL_MAX;  // error already flagged by the scan
-    int np2 = 1;
-    while (np2 < n) np2 <<= 1;
     unsigned long long* key = s_key[w];
     int* val = s_val[w];
+    if (n <= RANK_MAX) {
+        const int cl0 = P.col_cl_start[col];
+        const int ncl = min(P.col_ncl[col], COL_MAX / CL);
+        for (int k = lane; k < n; k += 32) {
+            const int s = P.col_atoms[start + k];
+            const unsigned int zb = lig_col ? 0u : __float_as_uint(P.xq_old[s].z);
+            key[k] = ((unsigned long long)zb << 32) | (unsigned int)P.orig_old[s];
+            val[k] = s;
+        }
+        __syncwarp();
+        // never outside the replica's own clusters (see below)
+        if (cl0 + ncl > R.cl_off + R.n_cl_cap || n > ncl * CL) return;
+        int* const perm = P.perm + cl0 * CL;
+        if (n <= 128) rank_column<4>(key, val, n, perm, lane);
+        else if (n <= 256) rank_column<8>(key, val, n, perm, lane);
+        else rank_column<16>(key, val, n, perm, lane);
+        for (int k = n + lane; k < ncl * CL; k += 32) perm[k] = -1;
+        for (int k = lane; k < ncl; k += 32) P.cl_col[cl0 + k] = col;
+        return;
+    }
+    int np2 = 1;
+    while (np2 < n) np2 <<= 1;
     for (int k = lane; k < np2; k += 32) {
         if (k < n) {
             const int s = P.col_atoms[start + k];
@@ -345,6 +392,7 @@ struct LBS {
     int hhead[HCAP];
     unsigned long long xm[XCAP][GM];
     int col_cs[MAXCOL], col_pref[MAXCOL + 1], col_k[MAXCOL];
+    int col_q[64];            // columns waiting for a full batch
     int n_e, n_x, overflow, n_col;
 };
 
@@ -600,20 +648,68 @@ __device__ __forceinline__ void lb_reset(L_t& L) {
     __syncwarp();
 }
 
-// Clusters of one column (n clusters sorted by z, z bounds zb[k] = (min, max))
-// whose z extent overlaps [wlo, whi]: the index range [a, b). Starts from the
-// index a uniform column would give and walks to the exact bounds; the bounds
-// are monotonic in k because the column is sorted by z.
+// Clusters of one column (n > 0 clusters sorted by z, z bounds zb[k] = (min,
+// max)) whose z extent overlaps [wlo, whi]: the index range [a, b). Starts from the
+// indexes a uniform column would give, reads four bounds around each at once
+// (their loads overlap; a walk's depend on each other) and walks on only where the
+// bound lies outside them; the bounds are monotonic in k because the column is
+// sorted by z.
 __device__ __forceinline__ void z_range(const float2* zb, int n, float wlo, float whi,
                                         float invLz, int& a_out, int& b_out) {
     int a = min(max((int)(wlo * invLz * n) - 1, 0), n);
-    while (a > 0 && zb[a - 1].y >= wlo) --a;
-    while (a < n && zb[a].y < wlo) ++a;
-    int b = min(max((int)(whi * invLz * n) + 2, a), n);
-    while (b < n && zb[b].x <= whi) ++b;
-    while (b > a && zb[b - 1].x > whi) --b;
+    int b = min(max((int)(whi * invLz * n) + 2, 0), n);
+    float ya[4], xb[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        ya[q] = zb[min(max(a - 2 + q, 0), n - 1)].y;
+        xb[q] = zb[min(max(b - 2 + q, 0), n - 1)].x;
+    }
+    // first k with max >= wlo
+    if (a > 0 && ya[1] >= wlo) {            // (ya[1]: cluster a - 1)
+        --a;
+        if (a > 0 && ya[0] >= wlo) {
+            --a;
+            while (a > 0 && zb[a - 1].y >= wlo) --a;
+        }
+    } else if (a < n && ya[2] < wlo) {      // (ya[2]: cluster a)
+        ++a;
+        if (a < n && ya[3] < wlo) {
+            ++a;
+            while (a < n && zb[a].y < wlo) ++a;
+        }
+    }
+    // last k with min <= whi, plus one
+    if (b < n && xb[2] <= whi) {            // (xb[2]: cluster b)
+        ++b;
+        if (b < n && xb[3] <= whi) {
+            ++b;
+            while (b < n && zb[b].x <= whi) ++b;
+        }
+    } else if (b > 0 && xb[1] > whi) {      // (xb[1]: cluster b - 1)
+        --b;
+        if (b > 0 && xb[0] > whi) {
+            --b;
+            while (b > 0 && zb[b - 1].x > whi) --b;
+        }
+    }
     a_out = a;
-    b_out = b;
+    b_out = max(a, b);
+}
+
+// Whether some cluster of [j0, j1) may belong to the lists of i-clusters [c, c +
+// ng) under the half-list rule (half_owner with n_wrap > 0): the forward cyclic
+// distance from an i-cluster grows along the range, so a range whose two ends both
+// lie in the half behind, without passing the i-cluster, is behind as a whole.
+__device__ __forceinline__ bool half_range(int c, int ng, int j0, int j1, int n_wrap) {
+    if (n_wrap <= 0) return true;
+    bool any = false;
+    for (int g = 0; g < ng; ++g) {
+        int d0 = j0 - (c + g), d1 = (j1 - 1) - (c + g);
+        if (d0 < 0) d0 += n_wrap;
+        if (d1 < 0) d1 += n_wrap;
+        any |= !(2 * d0 > n_wrap && d1 >= d0);
+    }
+    return any;
 }
 
 template <int G, int ECAP, int HCAP, int XCAP, int GM>
@@ -658,44 +754,81 @@ __device__ void build_group(const DevPtrs& P, LBS<ECAP, HCAP, XCAP, GM>& L, int 
         const float cwx = R.box[0] / R.ncx, cwy = R.box[1] / R.ncy;
         const float zlo = lo[2] - rl - ZSLACK, zhi = hi[2] + rl + ZSLACK;
         const float Lz = R.box[2], invLz = 1.0f / R.box[2];
-        for (int cb = 0; cb < ncand; cb += 32) {
-            // (a) segments of this batch of 32 columns: for each column that the
-            // group can reach in x/y and each z image, the range of its clusters
-            // (sorted by z) whose z extent overlaps the group's z window
+        // images kz with z_j + kz Lz in [zlo, zhi] for some z_j in [0, Lz) (most groups:
+        // one). With one image the order of the segments is that of the columns, so
+        // columns out of reach or on the wrong side of the half-list rule are
+        // dropped before the batches of 32 are formed.
+        int n_kz = 0;
+        for (int kz = -1; kz <= 1; ++kz) n_kz += zhi - kz * Lz >= 0.f && zlo - kz * Lz < Lz ? 1 : 0;
+        const int n_wrap = is_lig ? -1 : n_env;
+        int cb = 0, n_q = 0;   // next candidate column; columns waiting in the queue
+        while (cb < ncand || n_q > 0) {
+            // (a) segments of a batch of 32 columns: for each column that the group can
+            // reach in x/y and each z image, the range of its clusters (sorted by z)
+            // whose z extent overlaps the group's z window
             if (lane == 0) L.n_col = 0;
             __syncwarp();
             {
-                const int q = cb + lane;
-                bool ok = q < ncand;
-                int kx = 0, ky = 0, jcol = 0;
-                if (ok) {
-                    const int ix = ixlo + q / nyr, iy = iylo + q % nyr;
-                    kx = floor_div(ix, R.ncx);
-                    ky = floor_div(iy, R.ncy);
-                    const int wx = ix - kx * R.ncx, wy = iy - ky * R.ncy;
-                    // (1e-5 nm of slack keeps this coarse test more inclusive than the
-                    // exact bounding-box test under rounding)
-                    const float dxc = fmaxf(fmaxf(ix * cwx - hi[0], lo[0] - (ix + 1) * cwx) - 1e-5f, 0.f);
-                    const float dyc = fmaxf(fmaxf(iy * cwy - hi[1], lo[1] - (iy + 1) * cwy) - 1e-5f, 0.f);
-                    ok = kx >= -1 && kx <= 1 && ky >= -1 && ky <= 1 && dxc * dxc + dyc * dyc < rl2;
-                    jcol = R.col_off + wx * R.ncy + wy;
+                int key = -1;   // column | kx + 1 << 28 | ky + 1 << 30
+                while (cb < ncand && (n_kz > 1 ? n_q == 0 : n_q < 32)) {
+                    const int q = cb + lane;
+                    cb += 32;
+                    bool ok = q < ncand;
+                    int k = 0;
+                    if (ok) {
+                        const int ix = ixlo + q / nyr, iy = iylo + q % nyr;
+                        const int kx = floor_div(ix, R.ncx), ky = floor_div(iy, R.ncy);
+                        const int wx = ix - kx * R.ncx, wy = iy - ky * R.ncy;
+                        // (1e-5 nm of slack keeps this coarse test more inclusive than the
+                        // exact bounding-box test under rounding)
+                        const float dxc = fmaxf(fmaxf(ix * cwx - hi[0], lo[0] - (ix + 1) * cwx) - 1e-5f, 0.f);
+                        const float dyc = fmaxf(fmaxf(iy * cwy - hi[1], lo[1] - (iy + 1) * cwy) - 1e-5f, 0.f);
+                        ok = kx >= -1 && kx <= 1 && ky >= -1 && ky <= 1 && dxc * dxc + dyc * dyc < rl2;
+                        k = (wx * R.ncy + wy) | ((kx + 1) << 26) | ((ky + 1) << 28);
+                    }
+                    if (n_kz > 1) {   // this batch as it is
+                        key = ok ? k : -1;
+                        n_q = 32;
+                    } else {
+                        if (ok) {
+                            const int jcol = R.col_off + (k & 0x3FFFFFF);
+                            const int cs = P.col_cl_start[jcol], n = P.col_ncl[jcol];
+                            ok = n > 0 && half_range(c, ng, cs, cs + n, n_wrap);
+                        }
+                        const unsigned int bl = __ballot_sync(0xffffffffu, ok);
+                        if (ok) L.col_q[n_q + __popc(bl & ((1u << lane) - 1u))] = k;
+                        n_q += __popc(bl);
+                        __syncwarp();
+                    }
                 }
+                if (n_kz > 1) {
+                    n_q = 0;
+                } else {
+                    key = lane < n_q ? L.col_q[lane] : -1;
+                    const int rest = lane + 32 < n_q ? L.col_q[lane + 32] : 0;
+                    __syncwarp();
+                    if (lane + 32 < n_q) L.col_q[lane] = rest;
+                    n_q = max(0, n_q - 32);
+                    __syncwarp();
+                }
+                const bool ok = key >= 0;
+                const int jcol = R.col_off + (key & 0x3FFFFFF);
                 const int cs = ok ? P.col_cl_start[jcol] : 0;
                 const int n = ok ? P.col_ncl[jcol] : 0;
-#pragma unroll
+#pragma unroll 1
                 for (int kz = -1; kz <= 1; ++kz) {
                     // j clusters of image kz: z_j + kz Lz in [zlo, zhi], z_j in [0, Lz)
                     const float wlo = zlo - kz * Lz, whi = zhi - kz * Lz;
+                    if (!(whi >= 0.f && wlo < Lz)) continue;   // warp-uniform
                     int a = 0, b = 0;
-                    if (n > 0 && whi >= 0.f && wlo < Lz)
-                        z_range(P.clz + cs, n, fmaxf(wlo, 0.f), fminf(whi, Lz), invLz, a, b);
-                    const bool has = b > a;
+                    if (n > 0) z_range(P.clz + cs, n, fmaxf(wlo, 0.f), fminf(whi, Lz), invLz, a, b);
+                    const bool has = b > a && half_range(c, ng, cs + a, cs + b, n_wrap);
                     const unsigned int bl = __ballot_sync(0xffffffffu, has);
                     if (has) {
                         const int slot = L.n_col + __popc(bl & ((1u << lane) - 1u));
                         L.col_cs[slot] = cs + a;
                         L.col_pref[slot] = b - a;
-                        L.col_k[slot] = (kx + 1) | ((ky + 1) << 2) | ((kz + 1) << 4);
+                        L.col_k[slot] = ((key >> 26) & 15) | ((kz + 1) << 4);
                     }
                     __syncwarp();
                     if (lane == 0) L.n_col += __popc(bl);
@@ -748,8 +881,7 @@ __device__ void build_group(const DevPtrs& P, LBS<ECAP, HCAP, XCAP, GM>& L, int 
                 const float4 jb = jb_n, jh = jh_n;
                 if (t0 + 32 < T) fetch(t0 + 32 + lane, jc_n, kk_n, jb_n, jh_n);
                 const int kx = (kk & 3) - 1, ky = ((kk >> 2) & 3) - 1, kz = ((kk >> 4) & 3) - 1;
-                const int m = jb.w > 0.f ? lb_mask<G>(R, c, ng, bc, bh, jc, jb, jh, kx, ky, kz,
-                                                      is_lig ? -1 : n_env, rl2)
+                const int m = jb.w > 0.f ? lb_mask<G>(R, c, ng, bc, bh, jc, jb, jh, kx, ky, kz, n_wrap, rl2)
                                          : 0;
                 // up to 32 accepts follow: flush a buffer that might not hold them
                 __syncwarp();
@@ -802,6 +934,11 @@ constexpr int LIG_E = 1024, LIG_H = 1024, LIG_X = 128, LIG_WARPS = 2;
 // per SM (registers capped at 80): the few spills cost less than the latency
 // the extra warps hide (60.9 vs 66.8 ms per build of the 1,152-window batch
 // at the four blocks that 128 registers allow).
+// Bound by instruction issue and by the latency of the column and cluster bounds, so
+// what is out of reach or on the wrong side of the half-list rule is dropped before
+// batches are formed, and bounds are read side by side (24 windows of 25,000 atoms
+// 802 -> 664 us, 42 of 40,000 with 30 of 4,500 2629 -> 2184, one of 60,000 81 -> 60,
+// one of 4,500 37 -> 29).
 template <int G>
 __global__ void __launch_bounds__(ENV_WARPS * 32, 6) k_build_list_env(DevPtrs P, int chunk) {
     if (!P.cnt->rebuild) return;
@@ -1350,7 +1487,14 @@ static void launch_lb_env(const DevPtrs& P, cudaStream_t s) {
     k_build_list_env<G><<<grid, ENV_WARPS * 32, smem, s>>>(P, chunk);
 }
 
-void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl) {
+// s2, fork, join: a second stream and events for the ligand clusters' lists beside
+// the environment's (35 us of one warp's latency per cluster), or null
+void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl, cudaStream_t s2,
+                       cudaEvent_t fork, cudaEvent_t join) {
+    if (s2 && max_lig_cl > 0) {
+        cudaEventRecord(fork, s);
+        cudaStreamWaitEvent(s2, fork, 0);
+    }
     switch (P.group) {
         case 1: launch_lb_env<1>(P, s); break;
         case 2: launch_lb_env<2>(P, s); break;
@@ -1365,7 +1509,12 @@ void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl) {
             attr = true;
         }
         const int warps = P.R * max_lig_cl;
-        k_build_list_lig<<<(warps + LIG_WARPS - 1) / LIG_WARPS, LIG_WARPS * 32, smem, s>>>(P, max_lig_cl);
+        k_build_list_lig<<<(warps + LIG_WARPS - 1) / LIG_WARPS, LIG_WARPS * 32, smem, s2 ? s2 : s>>>(
+            P, max_lig_cl);
+        if (s2) {
+            cudaEventRecord(join, s2);
+            cudaStreamWaitEvent(s, join, 0);
+        }
     }
     k_build_prefix<<<1, 1024, 0, s>>>(P);
 }
