@@ -308,7 +308,7 @@ struct DevPtrs {
                                    // displacement of its atoms from its prune
                                    // positions > (prune_skin / 2)^2
     float beta, pbeta, nb2l2e, tbsp, sqrt_ke;
-    const float4* ewtab;           // [EW_NT] Coulomb force table (see ewald_table)
+    const float4* ewtab;           // [EW_NT] Coulomb force table, [EW_NT] erfc(beta r)
     int pme;                       // 1 = reciprocal-space Ewald terms are on
     const double2* pme_self;       // [systems] self energy of the environment / ligand charges
     float ewtab_inv_h;             // grid points per unit of r (nm^-1)

@@ -1253,7 +1253,8 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         // G''(r) = -(8 beta^3 / sqrt pi) r (1 - beta^2 r^2) e^{-beta^2 r^2}
         const double b = p->ewald_beta, tp = 2.0 / std::sqrt(M_PI);
         const double h = p->cutoff / (EW_NT - 1);
-        std::vector<float4> tab(EW_NT);
+        P.ewtab_inv_h = (float)(1.0 / h);
+        std::vector<float4> tab(2 * EW_NT);
         for (int j = 0; j < EW_NT; ++j) {
             const double r = j * h;
             const double e = std::exp(-b * b * r * r);
@@ -1262,18 +1263,31 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
             const double G2 = -4.0 * tp * b * b * b * r * (1.0 - b * b * r * r) * e;
             tab[j] = make_float4((float)G, (float)(G1 * h), (float)(0.5 * G2 * h * h), 0.f);
         }
-        float4* d_tab = dalloc<float4>(c, EW_NT, ok);
+        // erfc(beta r) for the energies, about the points that the kernel's binary32
+        // 1 / h names (the rounding of 1 / h would shift every energy the same way):
+        // value, slope, half the curvature, rounding of the value. The slope carries
+        // 3/16 of the cubic term (f^3 less its third Chebyshev polynomial on |f| <=
+        // 1/2), which leaves 1/32 of that: 8e-8 of erfc(3.6), 1e-9 of erfc(1).
+        const double he = 1.0 / (double)P.ewtab_inv_h;
+        for (int j = 0; j < EW_NT; ++j) {
+            const double r = j * he;
+            const double e = std::exp(-b * b * r * r), E0 = std::erfc(b * r);
+            const double E1 = -tp * b * e, E2 = 2.0 * tp * b * b * b * r * e,
+                         E3 = 2.0 * tp * b * b * b * (1.0 - 2.0 * b * b * r * r) * e;
+            tab[EW_NT + j] = make_float4((float)E0, (float)(E1 * he + E3 * he * he * he / 32.0),
+                                         (float)(0.5 * E2 * he * he), (float)(E0 - (double)(float)E0));
+        }
+        float4* d_tab = dalloc<float4>(c, 2 * EW_NT, ok);
         // on the context's stream, after the zero fill queued there by the
         // allocation (a copy on another stream could land before the fill)
         if (!ok ||
-            cudaMemcpyAsync(d_tab, tab.data(), sizeof(float4) * EW_NT, cudaMemcpyHostToDevice,
+            cudaMemcpyAsync(d_tab, tab.data(), sizeof(float4) * 2 * EW_NT, cudaMemcpyHostToDevice,
                             c->stream) != cudaSuccess ||
             cudaStreamSynchronize(c->stream) != cudaSuccess) {
             abfe_destroy(c);
             return set_error(nullptr, ABFE_ERR_OUT_OF_MEMORY, "Ewald table");
         }
         P.ewtab = d_tab;
-        P.ewtab_inv_h = (float)(1.0 / h);
     }
     P.drc2 = p->cutoff * p->cutoff;
     P.dbeta = p->ewald_beta;

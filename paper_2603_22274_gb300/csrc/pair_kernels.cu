@@ -42,7 +42,8 @@ struct Atom {
 template <typename T>
 struct KC {
     T rc2, beta, tbsp, nb2l2e, dke_sqrt;
-    const float4* tab;   // FP32 path: the Ewald force table in shared memory
+    const float4* tab;    // FP32 path: the Ewald force table in shared memory
+    const float4* etab;   // and that of erfc (energy steps)
     float inv_h;
 };
 
@@ -50,12 +51,12 @@ template <typename T>
 __device__ __forceinline__ KC<T> make_kc(const DevPtrs& P);
 template <>
 __device__ __forceinline__ KC<float> make_kc<float>(const DevPtrs& P) {
-    return KC<float>{P.rc2, P.beta, P.tbsp, P.nb2l2e, P.sqrt_ke, nullptr, P.ewtab_inv_h};
+    return KC<float>{P.rc2, P.beta, P.tbsp, P.nb2l2e, P.sqrt_ke, nullptr, nullptr, P.ewtab_inv_h};
 }
 template <>
 __device__ __forceinline__ KC<double> make_kc<double>(const DevPtrs& P) {
     return KC<double>{P.drc2, P.dbeta, 2.0 * P.dbeta / sqrt(3.14159265358979323846), 0.0,
-                      sqrt(P.dke), nullptr, 0.0f};
+                      sqrt(P.dke), nullptr, nullptr, 0.0f};
 }
 
 template <typename T>
@@ -106,6 +107,19 @@ __device__ __forceinline__ float ewald_G(float r, const float4* tab, float inv_h
     const float f = t - (tr - 12582912.0f);
     const float4 c = tab[j];
     return fmaf(fmaf(c.z, f, c.y), f, c.x);
+}
+
+// erfc(beta r) from its table, the centred quadratic about the nearest point of the
+// same grid (see ewald_G). The offset is one multiply-add, so r's own rounding is the
+// only one in it; the value at the point is held to twice binary32 (c.x + c.w), since
+// its rounding would be common to every pair near that point.
+__device__ __forceinline__ float ewald_erfc(float r, const float4* tab, float inv_h) {
+    const float t = fminf(r * inv_h, (float)(EW_NT - 1));
+    const float tr = t + 12582912.0f;
+    const int j = __float_as_int(tr) - 0x4B400000;
+    const float f = fmaf(r, inv_h, -(tr - 12582912.0f));
+    const float4 c = tab[j];
+    return c.x + fmaf(fmaf(c.z, f, c.y), f, c.w);
 }
 
 // correctly rounded / library-accurate variants, used where energies are
@@ -174,12 +188,27 @@ __device__ __forceinline__ void pair_env(const Atom<T>& ai, const Atom<T>& aj, b
     fi.x = fma(-fs, dx, fi.x); fi.y = fma(-fs, dy, fi.y); fi.z = fma(-fs, dz, fi.z);
     fj.x = fma(fs, dx, fj.x);  fj.y = fma(fs, dy, fj.y);  fj.z = fma(fs, dz, fj.z);
     if (ENERGY) {
-        // energies from correctly rounded arithmetic (energy steps only)
-        const T re = t_sqrt_acc(r2);
-        T erfc_e, ex_e;
-        ewald_acc(re, r2, K, erfc_e, ex_e);
-        const T vce = qq * erfc_e * t_rcp_acc(re);
-        const T s2e = sig * sig * t_rcp_acc(r2);
+        // (energy steps only)
+        T vce, r2inv;
+        if constexpr (sizeof(T) == 4) {
+            // The force's fast reciprocal root, corrected to r, 1 / r and 1 / r^2 of
+            // about half a unit in the last place each, and erfc from its table.
+            // sqrt, two reciprocals and erfcf, each accurate by itself, took 195
+            // issue cycles a pair, most of the pass (24 windows of 25,000 atoms:
+            // 1489 us with them, 750 us).
+            const float r0 = r2 * rinv;
+            const float re = fmaf(fmaf(-r0, r0, r2), 0.5f * rinv, r0);
+            const float y = fmaf(rinv, fmaf(-re, rinv, 1.f), rinv);
+            r2inv = fmaf(rinv2, fmaf(-r2, rinv2, 1.f), rinv2);
+            vce = qq * ewald_erfc(re, K.etab, K.inv_h) * y;
+        } else {
+            const T re = t_sqrt_acc(r2);
+            T erfc_e, ex_e;
+            ewald_acc(re, r2, K, erfc_e, ex_e);
+            vce = qq * erfc_e * t_rcp_acc(re);
+            r2inv = t_rcp_acc(r2);
+        }
+        const T s2e = sig * sig * r2inv;
         const T s6e = s2e * s2e * s2e;
         const T vlj = eps4 * fma(s6e, s6e, -s6e);
         elj += keep ? vlj : (T)0;
@@ -373,11 +402,12 @@ __device__ __forceinline__ void env_tail_row(const DevPtrs& P, const volatile in
 // where they are needed), so that 64 registers hold the round loop: with them in
 // registers it spilled inside the loop, which cost more than the atom of the
 // next round loaded ahead gained (24 x 25k atoms: 429 us with the prefetch, 472
-// with this claim scheme in registers too, 400 as it is).
+// with this claim scheme in registers too, 427 as it is).
 template <typename T, bool ENERGY, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     __shared__ float4 s_ewtab[sizeof(T) == 4 ? EW_NT : 1];
+    __shared__ float4 s_etab[sizeof(T) == 4 && ENERGY ? EW_NT : 1];
     // per warp and image code: u (0-26) and v (32-58) of the shifted j atom
     // relative to the i-cluster's reference atom
     __shared__ float4 s_shift[ENV_WARPS_MAX][64];
@@ -393,6 +423,10 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
         if constexpr (sizeof(T) == 4) {
             for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_ewtab[i] = P.ewtab[i];
             K.tab = s_ewtab;
+            if constexpr (ENERGY) {
+                for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_etab[i] = P.ewtab[EW_NT + i];
+                K.etab = s_etab;
+            }
         }
         if (lane == 0) {
             N[0] = w * (int)gridDim.x + (int)blockIdx.x;
@@ -920,7 +954,7 @@ void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precis
         if (energy) k_env_rows<float, true, 1><<<grid, block, 0, s>>>(P);
         else k_env_rows<float, false, 1><<<grid, block, 0, s>>>(P);
     } else {
-        if (energy) k_env_rows<float, true, 3><<<grid, block, 0, s>>>(P);
+        if (energy) k_env_rows<float, true, 4><<<grid, block, 0, s>>>(P);
         else k_env_rows<float, false, 4><<<grid, block, 0, s>>>(P);
     }
 }
@@ -930,7 +964,7 @@ int env_kernel_occupancy(int block, int precision, bool energy) {
     if (precision == 1)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<double, true, 2>, block, 0);
     else if (energy)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, true, 3>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, true, 4>, block, 0);
     else
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, false, 4>, block, 0);
     return nb;
