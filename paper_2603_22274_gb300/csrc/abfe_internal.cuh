@@ -46,6 +46,14 @@ constexpr int K_MAX = 256;
 // the separation vector. EW_NT points on r in [0, r_c]; point j holds
 // (G, G' h, G'' h^2 / 2) at r_j = j h for a centred quadratic in the offset.
 constexpr int EW_NT = 1024;
+// FP64 expansions of erfc(x) about x = j / ERFC_INV_H, j < ERFC_NT: eight Taylor
+// coefficients each (up to (x - x_j)^7)
+constexpr int ERFC_NT = 1025, ERFC_INV_H = 128;
+// FP64 pair kernels: warps per block and per item of the row kernel, idle lanes that
+// make it refill, warps per item of the ligand kernel (12 frames of 672 atoms: row
+// kernel's 1, 2, 4, 8 per item 501, 476, 550, 608 us a pass; refills at 4, 8, 12 idle
+// lanes 502, 502, 511; ligand kernel's 1, 2, 4 per item 476, 458, 457)
+constexpr int ENVD_WARPS = 4, ENVD_SEG = 2, ENVD_REFILL = 8, LIGD_SEG = 2;
 constexpr int COL_MAX = 1024;       // atoms per column (per-column sort capacity)
 constexpr double FSCALE = 4294967296.0;
 constexpr float FSCALEF = 4294967296.0f;
@@ -311,6 +319,7 @@ struct DevPtrs {
     const float4* ewtab;           // [EW_NT] Coulomb force table, [EW_NT] erfc(beta r)
     int pme;                       // 1 = reciprocal-space Ewald terms are on
     const double2* pme_self;       // [systems] self energy of the environment / ligand charges
+    const double2* erfc_tab;       // [ERFC_NT][4] erfc's expansions (FP64 contexts)
     float ewtab_inv_h;             // grid points per unit of r (nm^-1)
     double drc2, dbeta, dke;
     int group, max_entries, ligand_mode;

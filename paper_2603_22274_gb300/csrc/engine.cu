@@ -625,11 +625,12 @@ void update_grids(abfe_ctx* c) {
     // kernels claim what is left over): blocks without work still took registers
     // from the kernels beside them (one solvent window: 53 us of pair kernel next to
     // its forked neighbours, 37 alone)
-    const int warps = c->tune.block_threads / 32;
-    const int64_t items = (int64_t)c->C * (1 + c->epc_max / c->tune.max_entries);
+    const bool f64 = c->prm.precision == 1;
+    const int warps = f64 ? ENVD_WARPS : c->tune.block_threads / 32;
+    const int64_t items = (int64_t)c->C * (1 + c->epc_max / c->tune.max_entries) * (f64 ? ENVD_SEG : 1);
     c->env_grid = (int)std::min<int64_t>((int64_t)c->n_sm * occ,
                                          std::max<int64_t>(c->n_sm, (items + warps - 1) / warps));
-    const int64_t lig_items = (int64_t)c->n_lig_cl * (1 + 2 * c->epc_max / LIG_CHUNK);
+    const int64_t lig_items = (int64_t)c->n_lig_cl * (1 + 2 * c->epc_max / LIG_CHUNK) * (f64 ? LIGD_SEG : 1);
     c->lig_grid = (int)std::min<int64_t>(c->n_sm * 4, std::max<int64_t>(1, (lig_items + 3) / 4));
     c->P.group = c->prm.precision == 1 ? 1 : c->tune.group;
     c->P.max_entries = c->tune.max_entries;
@@ -881,7 +882,7 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         for (int i = 0; i < n; ++i) {
             h_prm.push_back(make_float4((float)(d.charge[i] * sqke), (float)(0.5 * d.sigma[i]),
                                         (float)(2.0 * std::sqrt(d.epsilon[i])), (float)(1.0 / d.mass[i])));
-            h_prmd.push_back(dbl4{d.charge[i], d.sigma[i], d.epsilon[i], 1.0 / d.mass[i]});
+            h_prmd.push_back(dbl4{d.charge[i], 0.5 * d.sigma[i], 2.0 * std::sqrt(d.epsilon[i]), 1.0 / d.mass[i]});
             h_lig.push_back(d.is_ligand[i] ? 1 : 0);
             nl += d.is_ligand[i] ? 1 : 0;
         }
@@ -1288,6 +1289,31 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
             return set_error(nullptr, ABFE_ERR_OUT_OF_MEMORY, "Ewald table");
         }
         P.ewtab = d_tab;
+        if (p->precision == 1) {
+            // erfc's Taylor coefficients from those of g = exp(-x^2), whose derivative
+            // is -2 x g: (n + 1) g_{n+1} = -2 (x_j g_n + g_{n-1})
+            std::vector<double> et((size_t)ERFC_NT * 8);
+            for (int j = 0; j < ERFC_NT; ++j) {
+                const double x = (double)j / ERFC_INV_H;
+                double* t = et.data() + (size_t)j * 8;
+                double g0 = 0.0, g1 = std::exp(-x * x);
+                t[0] = std::erfc(x);
+                for (int n = 0; n < 7; ++n) {
+                    t[n + 1] = -tp * g1 / (n + 1);
+                    const double g2 = -2.0 * (x * g1 + g0) / (n + 1);
+                    g0 = g1;
+                    g1 = g2;
+                }
+            }
+            double2* d_et = dalloc<double2>(c, et.size() / 2, ok);
+            if (!ok || cudaMemcpyAsync(d_et, et.data(), sizeof(double) * et.size(), cudaMemcpyHostToDevice,
+                                       c->stream) != cudaSuccess ||
+                cudaStreamSynchronize(c->stream) != cudaSuccess) {
+                abfe_destroy(c);
+                return set_error(nullptr, ABFE_ERR_OUT_OF_MEMORY, "erfc table");
+            }
+            P.erfc_tab = d_et;
+        }
     }
     P.drc2 = p->cutoff * p->cutoff;
     P.dbeta = p->ewald_beta;

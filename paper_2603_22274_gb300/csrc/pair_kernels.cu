@@ -44,6 +44,7 @@ struct KC {
     T rc2, beta, tbsp, nb2l2e, dke_sqrt;
     const float4* tab;    // FP32 path: the Ewald force table in shared memory
     const float4* etab;   // and that of erfc (energy steps)
+    const double2* dtab;  // FP64 path: erfc's expansions (see erfc_table)
     float inv_h;
 };
 
@@ -51,12 +52,12 @@ template <typename T>
 __device__ __forceinline__ KC<T> make_kc(const DevPtrs& P);
 template <>
 __device__ __forceinline__ KC<float> make_kc<float>(const DevPtrs& P) {
-    return KC<float>{P.rc2, P.beta, P.tbsp, P.nb2l2e, P.sqrt_ke, nullptr, nullptr, P.ewtab_inv_h};
+    return KC<float>{P.rc2, P.beta, P.tbsp, P.nb2l2e, P.sqrt_ke, nullptr, nullptr, nullptr, P.ewtab_inv_h};
 }
 template <>
 __device__ __forceinline__ KC<double> make_kc<double>(const DevPtrs& P) {
     return KC<double>{P.drc2, P.dbeta, 2.0 * P.dbeta / sqrt(3.14159265358979323846), 0.0,
-                      sqrt(P.dke), nullptr, nullptr, 0.0f};
+                      sqrt(P.dke), nullptr, nullptr, P.erfc_tab, 0.0f};
 }
 
 template <typename T>
@@ -80,20 +81,37 @@ __device__ __forceinline__ Atom<double> load_atom<double>(const DevPtrs& P, int 
         const dbl4 p = P.sys_prmd[sys_atom_off + o];
         // alchemical oxygens: q0 + (1 - lambda_q) dq
         a.q = fma(1.0 - R.dlam_q, P.sys_dqd[sys_atom_off + o], p.x) * K.dke_sqrt;
-        a.sh = 0.5 * p.y;
-        a.e2 = 2.0 * sqrt(p.z);
+        a.sh = p.y;
+        a.e2 = p.z;
     }
     return a;
 }
 
-__device__ __forceinline__ float t_rsqrt(float x) { return rsqrt_fast(x); }
-__device__ __forceinline__ double t_rsqrt(double x) { return rsqrt(x); }
 
-// erfc(beta r) and exp(-beta^2 r^2)
-__device__ __forceinline__ void ewald(double r, double r2, const KC<double>& K, double& erfcv,
-                                      double& ex) {
-    ex = exp(-K.beta * K.beta * r2);
-    erfcv = erfc(K.beta * r);
+// erfc(x) and its derivative from the expansions about multiples of 1 / 128 (x >= 0;
+// beyond the last point, 8, the value there: 1e-29). Thirteen multiply-adds and two
+// loads' latency where erfc and exp together take over 4,000 issue cycles of the FP64
+// pipe per warp; the remainder is below 1e-16 of the value up to x = 5 and of 1e-13
+// everywhere.
+__device__ __forceinline__ void erfc_table(double x, const double2* tab, double& e, double& d) {
+    const double t = fma(x, (double)ERFC_INV_H, 6755399441055744.0);   // 1.5 * 2^52: rounds to an integer
+    const unsigned int j = min((unsigned int)__double2loint(t), (unsigned int)(ERFC_NT - 1));
+    const double f = fma(t - 6755399441055744.0, -1.0 / ERFC_INV_H, x);
+    const double2* c = tab + (size_t)j * 4;
+    const double2 c67 = c[3], c45 = c[2], c23 = c[1], c01 = c[0];
+    double p = fma(c67.y, f, c67.x);
+    double q = fma(c67.y, f, p);
+    p = fma(p, f, c45.y);
+    q = fma(q, f, p);
+    p = fma(p, f, c45.x);
+    q = fma(q, f, p);
+    p = fma(p, f, c23.y);
+    q = fma(q, f, p);
+    p = fma(p, f, c23.x);
+    q = fma(q, f, p);
+    p = fma(p, f, c01.y);
+    d = fma(q, f, p);
+    e = fma(p, f, c01.x);
 }
 
 // G(r) from the shared-memory table: the nearest grid point j = round(t),
@@ -125,7 +143,6 @@ __device__ __forceinline__ float ewald_erfc(float r, const float4* tab, float in
 // correctly rounded / library-accurate variants, used where energies are
 // summed for dU/dlambda and u_kn (ligand pairs, energy steps)
 __device__ __forceinline__ float t_sqrt_acc(float x) { return __fsqrt_rn(x); }
-__device__ __forceinline__ double t_sqrt_acc(double x) { return sqrt(x); }
 __device__ __forceinline__ float t_rcp_acc(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double t_rcp_acc(double x) { return 1.0 / x; }
 __device__ __forceinline__ void ewald_acc(float r, float r2, const KC<float>& K, float& erfcv,
@@ -133,9 +150,24 @@ __device__ __forceinline__ void ewald_acc(float r, float r2, const KC<float>& K,
     ex = expf(-(K.beta * K.beta) * r2);
     erfcv = erfcf(K.beta * r);
 }
-__device__ __forceinline__ void ewald_acc(double r, double r2, const KC<double>& K, double& erfcv,
+__device__ __forceinline__ void ewald_acc(double r, double, const KC<double>& K, double& erfcv,
                                           double& ex) {
-    ewald(r, r2, K, erfcv, ex);
+    double d;   // erfc'(x) = -2 / sqrt(pi) exp(-x^2)
+    erfc_table(K.beta * r, K.dtab, erfcv, d);
+    ex = -0.88622692545275801 * d;
+}
+
+// r, 1 / r and 1 / r^2: for energies and ligand pairs
+__device__ __forceinline__ void root_acc(float r2, float& r, float& rinv, float& rinv2) {
+    r = t_sqrt_acc(r2);
+    rinv = t_rcp_acc(r);
+    rinv2 = t_rcp_acc(r2);
+}
+__device__ __forceinline__ void root_acc(double r2, double& r, double& rinv, double& rinv2) {
+    rinv = rsqrt(r2);
+    const double r0 = r2 * rinv;
+    r = fma(fma(-r0, r0, r2), 0.5 * rinv, r0);
+    rinv2 = rinv * rinv;
 }
 
 // x_j + s - c (image shift s, reference atom c of the i-cluster): the box
@@ -157,62 +189,44 @@ __device__ __forceinline__ const RowItem& row_item(const DevPtrs& P, int it) {
 
 // ------------------------------------------------------------------ env pair
 // (a pair that is not kept adds exact zeros)
-template <typename T, bool ENERGY>
-__device__ __forceinline__ void pair_env(const Atom<T>& ai, const Atom<T>& aj, bool keep,
-                                         T3<T>& fi, T3<T>& fj, T& elj, T& ec, const KC<T>& K) {
-    const T dx = aj.x - ai.x, dy = aj.y - ai.y, dz = aj.z - ai.z;
-    const T r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+template <bool ENERGY>
+__device__ __forceinline__ void pair_env(const Atom<float>& ai, const Atom<float>& aj, bool keep,
+                                         T3<float>& fi, T3<float>& fj, float& elj, float& ec,
+                                         const KC<float>& K) {
+    const float dx = aj.x - ai.x, dy = aj.y - ai.y, dz = aj.z - ai.z;
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
     keep = keep && (r2 < K.rc2);
-    const T rinv = t_rsqrt(r2);
-    const T rinv2 = rinv * rinv;
-    const T qq = ai.q * aj.q;
-    T fcr;  // Coulomb force times r^2
-    if constexpr (sizeof(T) == 4) {
-        // Coulomb force qq G(r) / r^3 from the table
-        fcr = qq * ewald_G(r2 * rinv, K.tab, K.inv_h) * rinv;
-    } else {
-        const T r = r2 * rinv;
-        T erfcv, ex;
-        ewald(r, r2, K, erfcv, ex);
-        const T vc = qq * erfcv * rinv;
-        fcr = fma(qq * K.tbsp, ex, vc);
-    }
-    const T sig = ai.sh + aj.sh;
-    const T eps4 = ai.e2 * aj.e2;
-    const T s2 = sig * sig * rinv2;
-    const T s6 = s2 * s2 * s2;
+    const float rinv = rsqrt_fast(r2);
+    const float rinv2 = rinv * rinv;
+    const float qq = ai.q * aj.q;
+    // Coulomb force times r^2: qq G(r) / r from the table
+    const float fcr = qq * ewald_G(r2 * rinv, K.tab, K.inv_h) * rinv;
+    const float sig = ai.sh + aj.sh;
+    const float eps4 = ai.e2 * aj.e2;
+    const float s2 = sig * sig * rinv2;
+    const float s6 = s2 * s2 * s2;
     // F / r = [Coulomb r^2 + 4 eps s6 (12 s6 - 6)] / r^2
-    const T fs = keep ? fma(eps4 * s6, fma((T)12, s6, (T)-6), fcr) * rinv2 : (T)0;
+    const float fs = keep ? fmaf(eps4 * s6, fmaf(12.f, s6, -6.f), fcr) * rinv2 : 0.f;
     // explicit FMAs (never left to contraction), so the force and energy
     // variants of the kernel add every pair force with the same roundings
-    fi.x = fma(-fs, dx, fi.x); fi.y = fma(-fs, dy, fi.y); fi.z = fma(-fs, dz, fi.z);
-    fj.x = fma(fs, dx, fj.x);  fj.y = fma(fs, dy, fj.y);  fj.z = fma(fs, dz, fj.z);
+    fi.x = fmaf(-fs, dx, fi.x); fi.y = fmaf(-fs, dy, fi.y); fi.z = fmaf(-fs, dz, fi.z);
+    fj.x = fmaf(fs, dx, fj.x);  fj.y = fmaf(fs, dy, fj.y);  fj.z = fmaf(fs, dz, fj.z);
     if (ENERGY) {
-        // (energy steps only)
-        T vce, r2inv;
-        if constexpr (sizeof(T) == 4) {
-            // The force's fast reciprocal root, corrected to r, 1 / r and 1 / r^2 of
-            // about half a unit in the last place each, and erfc from its table.
-            // sqrt, two reciprocals and erfcf, each accurate by itself, took 195
-            // issue cycles a pair, most of the pass (24 windows of 25,000 atoms:
-            // 1489 us with them, 750 us).
-            const float r0 = r2 * rinv;
-            const float re = fmaf(fmaf(-r0, r0, r2), 0.5f * rinv, r0);
-            const float y = fmaf(rinv, fmaf(-re, rinv, 1.f), rinv);
-            r2inv = fmaf(rinv2, fmaf(-r2, rinv2, 1.f), rinv2);
-            vce = qq * ewald_erfc(re, K.etab, K.inv_h) * y;
-        } else {
-            const T re = t_sqrt_acc(r2);
-            T erfc_e, ex_e;
-            ewald_acc(re, r2, K, erfc_e, ex_e);
-            vce = qq * erfc_e * t_rcp_acc(re);
-            r2inv = t_rcp_acc(r2);
-        }
-        const T s2e = sig * sig * r2inv;
-        const T s6e = s2e * s2e * s2e;
-        const T vlj = eps4 * fma(s6e, s6e, -s6e);
-        elj += keep ? vlj : (T)0;
-        ec += keep ? vce : (T)0;
+        // (energy steps only.) The force's fast reciprocal root, corrected to r, 1 / r
+        // and 1 / r^2 of about half a unit in the last place each, and erfc from its
+        // table. sqrt, two reciprocals and erfcf, each accurate by itself, took 195
+        // issue cycles a pair, most of the pass (24 windows of 25,000 atoms: 1489 us
+        // with them, 750 us).
+        const float r0 = r2 * rinv;
+        const float re = fmaf(fmaf(-r0, r0, r2), 0.5f * rinv, r0);
+        const float y = fmaf(rinv, fmaf(-re, rinv, 1.f), rinv);
+        const float r2inv = fmaf(rinv2, fmaf(-r2, rinv2, 1.f), rinv2);
+        const float vce = qq * ewald_erfc(re, K.etab, K.inv_h) * y;
+        const float s2e = sig * sig * r2inv;
+        const float s6e = s2e * s2e * s2e;
+        const float vlj = eps4 * fmaf(s6e, s6e, -s6e);
+        elj += keep ? vlj : 0.f;
+        ec += keep ? vce : 0.f;
     }
 }
 
@@ -310,65 +324,70 @@ __device__ __forceinline__ int warp_sum_24(T (&v)[24], int lane) {
 constexpr int ENV_WARPS_MAX = 8;
 
 // one i atom in shared memory: x, y, z, q sqrt(ke), sigma/2, 2 sqrt(eps), -, -
-template <typename T>
-__device__ __forceinline__ Atom<T> ld_iatom(const T* p);
-template <>
-__device__ __forceinline__ Atom<float> ld_iatom<float>(const float* p) {
+__device__ __forceinline__ Atom<float> ld_iatom(const float* p) {
     const float4 a = reinterpret_cast<const float4*>(p)[0];
     const float2 b = reinterpret_cast<const float2*>(p)[2];
     return Atom<float>{a.x, a.y, a.z, a.w, b.x, b.y};
 }
-template <>
-__device__ __forceinline__ Atom<double> ld_iatom<double>(const double* p) {
-    const double2 a = reinterpret_cast<const double2*>(p)[0];
-    const double2 b = reinterpret_cast<const double2*>(p)[1];
-    const double2 c = reinterpret_cast<const double2*>(p)[2];
-    return Atom<double>{a.x, a.y, b.x, b.y, c.x, c.y};
-}
-template <typename T>
-__device__ __forceinline__ void st_iatom(T* p, const Atom<T>& a) {
+__device__ __forceinline__ void st_iatom(float* p, const Atom<float>& a) {
     p[0] = a.x; p[1] = a.y; p[2] = a.z; p[3] = a.q; p[4] = a.sh; p[5] = a.e2;
-    p[6] = (T)0; p[7] = (T)0;
+    p[6] = 0.f; p[7] = 0.f;
 }
 
 // adds a force component to an accumulator unless it is zero (no pair in range)
-template <typename T>
-__device__ __forceinline__ void red_nonzero(long long* p, T f) {
-    const long long v = sizeof(T) == 8 ? to_fixed_d((double)f) : to_fixed((float)f);
-    if (f != (T)0) add_fixed(p, v);
+__device__ __forceinline__ void red_nonzero(long long* p, float f) {
+    const long long v = to_fixed(f);
+    if (f != 0.f) add_fixed(p, v);
+}
+__device__ __forceinline__ void red_nonzero(long long* p, double f) {
+    const long long v = to_fixed_d(f);
+    if (v != 0) add_fixed(p, v);
+}
+
+// Image shifts of a replica's box, by code, for the lane's code: x_j + s - c for image
+// shift s and reference atom c is evaluated as (x_j + u) - v with u = s - c, v = 0
+// where s > 0 (then c lies near the box length, and s - c is exact) and u = s, v = c
+// otherwise (x_j + s is exact where s < 0, x_j lying near the box length): no box-sized
+// sum is rounded.
+__device__ __forceinline__ void row_shifts(const RepDev& R, const float4& c, int lane, float4* sh) {
+    if (lane < 27) {
+        const float sx = (float)(lane % 3 - 1) * R.box[0],
+                    sy = (float)((lane / 3) % 3 - 1) * R.box[1],
+                    sz = (float)(lane / 9 - 1) * R.box[2];
+        sh[lane] = make_float4(sx > 0.f ? sx - c.x : sx, sy > 0.f ? sy - c.y : sy,
+                               sz > 0.f ? sz - c.z : sz, 0.f);
+        sh[32 + lane] = make_float4(sx > 0.f ? 0.f : c.x, sy > 0.f ? 0.f : c.y,
+                                    sz > 0.f ? 0.f : c.z, 0.f);
+    }
 }
 
 // One row of a lane against the i atoms; CHECK: minus those in `em`.
-template <typename T, bool ENERGY, bool CHECK>
-__device__ __forceinline__ void env_row(const DevPtrs& P, const KC<T>& K, const T* s_ia,
+template <bool ENERGY, bool CHECK>
+__device__ __forceinline__ void env_row(const DevPtrs& P, const KC<float>& K, const float* s_ia,
                                         const float4* sh, unsigned int word, unsigned int em,
-                                        const Atom<T>& aj, T3<T> (&fi)[CL], double& elj_d,
+                                        const Atom<float>& aj, T3<float> (&fi)[CL], double& elj_d,
                                         double& ec_d) {
     // the j atom relative to the cluster's reference atom c, (x_j + u) - v
     // with (u, v) from the row's image code
     const int code = (int)(word >> ROW_SLOT_BITS);
     const float4 u = sh[code], v = sh[32 + code];
-    Atom<T> a = aj;
-    a.x = ((T)aj.x + (T)u.x) - (T)v.x;
-    a.y = ((T)aj.y + (T)u.y) - (T)v.y;
-    a.z = ((T)aj.z + (T)u.z) - (T)v.z;
-    T3<T> fj{(T)0, (T)0, (T)0};
-    T elj = 0, ec = 0;
+    Atom<float> a = aj;
+    a.x = (aj.x + u.x) - v.x;
+    a.y = (aj.y + u.y) - v.y;
+    a.z = (aj.z + u.z) - v.z;
+    T3<float> fj{0.f, 0.f, 0.f};
+    float elj = 0, ec = 0;
 #pragma unroll
-    for (int ii = 0; ii < CL; ++ii) {
-        // (FP64: skipped rather than evaluated and dropped)
-        if (CHECK && sizeof(T) == 8 && ((em >> ii) & 1u)) continue;
-        pair_env<T, ENERGY>(ld_iatom<T>(s_ia + ii * 8), a, !(CHECK && ((em >> ii) & 1u)), fi[ii], fj,
-                            elj, ec, K);
-    }
+    for (int ii = 0; ii < CL; ++ii)
+        pair_env<ENERGY>(ld_iatom(s_ia + ii * 8), a, !(CHECK && ((em >> ii) & 1u)), fi[ii], fj, elj, ec, K);
     if (ENERGY) {
         elj_d += (double)elj;
         ec_d += (double)ec;
     }
     const int ja = (int)(word & ROW_SLOT_MASK);
-    red_nonzero<T>(P.fx + ja, fj.x);
-    red_nonzero<T>(P.fy + ja, fj.y);
-    red_nonzero<T>(P.fz + ja, fj.z);
+    red_nonzero(P.fx + ja, fj.x);
+    red_nonzero(P.fy + ja, fj.y);
+    red_nonzero(P.fz + ja, fj.z);
 }
 
 // row k of an item (I: the words of a RowItem) beyond its full rounds: plain
@@ -403,30 +422,28 @@ __device__ __forceinline__ void env_tail_row(const DevPtrs& P, const volatile in
 // registers it spilled inside the loop, which cost more than the atom of the
 // next round loaded ahead gained (24 x 25k atoms: 429 us with the prefetch, 472
 // with this claim scheme in registers too, 427 as it is).
-template <typename T, bool ENERGY, int MINB>
+template <bool ENERGY, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __shared__ float4 s_ewtab[sizeof(T) == 4 ? EW_NT : 1];
-    __shared__ float4 s_etab[sizeof(T) == 4 && ENERGY ? EW_NT : 1];
+    __shared__ float4 s_ewtab[EW_NT];
+    __shared__ float4 s_etab[ENERGY ? EW_NT : 1];
     // per warp and image code: u (0-26) and v (32-58) of the shifted j atom
     // relative to the i-cluster's reference atom
     __shared__ float4 s_shift[ENV_WARPS_MAX][64];
-    __shared__ __align__(16) T s_iat[ENV_WARPS_MAX][CL * 8];
+    __shared__ __align__(16) float s_iat[ENV_WARPS_MAX][CL * 8];
     __shared__ int s_item[ENV_WARPS_MAX][8];   // the warp's RowItem
     __shared__ int s_next[ENV_WARPS_MAX][2];   // its next item, end of the claimed ones
     volatile int* const I = s_item[w];
     volatile int* const N = s_next[w];
-    KC<T> K = make_kc<T>(P);
+    KC<float> K = make_kc<float>(P);
     {
         const int n_items = P.ritem_pref[P.R];
         if ((int)blockIdx.x >= n_items) return;   // no warp of this block has an item
-        if constexpr (sizeof(T) == 4) {
-            for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_ewtab[i] = P.ewtab[i];
-            K.tab = s_ewtab;
-            if constexpr (ENERGY) {
-                for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_etab[i] = P.ewtab[EW_NT + i];
-                K.etab = s_etab;
-            }
+        for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_ewtab[i] = P.ewtab[i];
+        K.tab = s_ewtab;
+        if constexpr (ENERGY) {
+            for (int i = threadIdx.x; i < EW_NT; i += blockDim.x) s_etab[i] = P.ewtab[EW_NT + i];
+            K.etab = s_etab;
         }
         if (lane == 0) {
             N[0] = w * (int)gridDim.x + (int)blockIdx.x;
@@ -435,7 +452,7 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
         __syncthreads();
     }
     float4* const sh = s_shift[w];
-    T* const s_ia = s_iat[w];
+    float* const s_ia = s_iat[w];
     for (;;) {
         {
             __syncwarp();
@@ -455,38 +472,25 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
             const RowItem& item = row_item(P, it);
             if (lane < 8) I[lane] = reinterpret_cast<const int*>(&item)[lane];
             __syncwarp();
-            // image shifts of this replica's box, by code; the i-cluster's atoms
-            // relative to its first atom (the reference c; same cluster: exact)
-            // x_j + s - c for image shift s is evaluated as (x_j + u) - v with
-            // u = s - c, v = 0 where s > 0 (then c lies near the box length, and
-            // s - c is exact) and u = s, v = c otherwise (x_j + s is exact where
-            // s < 0, x_j lying near the box length): no box-sized sum is rounded
+            // image shifts; the i-cluster's atoms relative to its first atom (the
+            // reference c; same cluster: exact)
             const RepDev& R = P.reps[P.rep_of_cl[I[0]]];
             const float4 c = P.xq[I[0] * CL];
-            if (lane < 27) {
-                const float sx = (float)(lane % 3 - 1) * R.box[0],
-                            sy = (float)((lane / 3) % 3 - 1) * R.box[1],
-                            sz = (float)(lane / 9 - 1) * R.box[2];
-                sh[lane] = make_float4(sx > 0.f ? sx - c.x : sx, sy > 0.f ? sy - c.y : sy,
-                                       sz > 0.f ? sz - c.z : sz, 0.f);
-                sh[32 + lane] = make_float4(sx > 0.f ? 0.f : c.x, sy > 0.f ? 0.f : c.y,
-                                            sz > 0.f ? 0.f : c.z, 0.f);
-            }
+            row_shifts(R, c, lane, sh);
             if (lane < CL) {
-                Atom<T> ai = load_atom<T>(P, I[0] * CL + lane, R, K);
-                ai.x -= (T)c.x;
-                ai.y -= (T)c.y;
-                ai.z -= (T)c.z;
-                st_iatom<T>(s_ia + lane * 8, ai);
+                Atom<float> ai = load_atom<float>(P, I[0] * CL + lane, R, K);
+                ai.x -= c.x;
+                ai.y -= c.y;
+                ai.z -= c.z;
+                st_iatom(s_ia + lane * 8, ai);
             }
             __syncwarp();
         }
-        T3<T> fi[CL];
+        T3<float> fi[CL];
 #pragma unroll
-        for (int ii = 0; ii < CL; ++ii) fi[ii] = T3<T>{(T)0, (T)0, (T)0};
+        for (int ii = 0; ii < CL; ++ii) fi[ii] = T3<float>{0.f, 0.f, 0.f};
         double elj = 0.0, ec = 0.0;
-        // FP64 parameters are looked up per replica
-        const RepDev& R = P.reps[sizeof(T) == 8 ? P.rep_of_cl[I[0]] : 0];
+        const RepDev& R = P.reps[0];   // (FP32 atoms hold their own parameters)
         {
             // full rounds: the next round's row word is loaded a round ahead, its atom
             // is not (the other warps cover that latency at fewer registers) unless
@@ -495,17 +499,17 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
             const unsigned int* rp = P.rows + ((unsigned int)I[1] + (unsigned int)lane);
             unsigned int word = nf > 0 ? *rp : 0u;
             if (MINB == 1) {
-                Atom<T> aj{};
-                if (nf > 0) aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
+                Atom<float> aj{};
+                if (nf > 0) aj = load_atom<float>(P, (int)(word & ROW_SLOT_MASK), R, K);
                 for (; nf > 0; --nf) {
                     rp += 32;
                     unsigned int word_n = word;
-                    Atom<T> aj_n = aj;
+                    Atom<float> aj_n = aj;
                     if (nf > 1) {
                         word_n = *rp;
-                        aj_n = load_atom<T>(P, (int)(word_n & ROW_SLOT_MASK), R, K);
+                        aj_n = load_atom<float>(P, (int)(word_n & ROW_SLOT_MASK), R, K);
                     }
-                    env_row<T, ENERGY, false>(P, K, s_ia, sh, word, 0u, aj, fi, elj, ec);
+                    env_row<ENERGY, false>(P, K, s_ia, sh, word, 0u, aj, fi, elj, ec);
                     word = word_n;
                     aj = aj_n;
                 }
@@ -513,8 +517,8 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
                 for (; nf > 0; --nf) {
                     rp += 32;
                     const unsigned int word_n = nf > 1 ? *rp : 0u;
-                    const Atom<T> aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
-                    env_row<T, ENERGY, false>(P, K, s_ia, sh, word, 0u, aj, fi, elj, ec);
+                    const Atom<float> aj = load_atom<float>(P, (int)(word & ROW_SLOT_MASK), R, K);
+                    env_row<ENERGY, false>(P, K, s_ia, sh, word, 0u, aj, fi, elj, ec);
                     word = word_n;
                 }
             }
@@ -522,25 +526,24 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
         for (int k0 = (I[3] & 0xFFFF) & ~31; k0 < (I[3] & 0xFFFF) + I[4] + I[5] + (I[3] >> 16); k0 += 32) {
             unsigned int word, em;
             env_tail_row(P, I, k0 + lane, word, em);
-            const Atom<T> aj = load_atom<T>(P, (int)(word & ROW_SLOT_MASK), R, K);
-            env_row<T, ENERGY, true>(P, K, s_ia, sh, word, em, aj, fi, elj, ec);
+            const Atom<float> aj = load_atom<float>(P, (int)(word & ROW_SLOT_MASK), R, K);
+            env_row<ENERGY, true>(P, K, s_ia, sh, word, em, aj, fi, elj, ec);
         }
         // i forces: the 24 values 3 ii + c summed over the warp (transposed);
         // value v ends on the four lanes of group v / 3, and the lane with
         // lane % 4 == v % 3 < 3 writes it
-        T v[3 * CL];
+        float v[3 * CL];
 #pragma unroll
         for (int ii = 0; ii < CL; ++ii) {
             v[3 * ii] = fi[ii].x;
             v[3 * ii + 1] = fi[ii].y;
             v[3 * ii + 2] = fi[ii].z;
         }
-        const int vi = warp_sum_24<T>(v, lane);
-        if ((lane & 3) < 3 && v[0] != (T)0) {
+        const int vi = warp_sum_24<float>(v, lane);
+        if ((lane & 3) < 3 && v[0] != 0.f) {
             const int c = vi % 3;
             long long* d = c == 0 ? P.fx : (c == 1 ? P.fy : P.fz);
-            add_fixed(d + I[0] * CL + vi / 3,
-                      (sizeof(T) == 4) ? to_fixed((float)v[0]) : to_fixed_d((double)v[0]));
+            add_fixed(d + I[0] * CL + vi / 3, to_fixed(v[0]));
         }
         if (ENERGY) {
             const double sl = warp_sum<double>(elj);
@@ -552,6 +555,152 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
                 add_fixed(P.eacc + (size_t)rep * EA_N + EA_ENV_C, to_fixed_d(sc));
             }
         }
+    }
+}
+
+// FP64 environment rows (precision 1: energies on every pass), bound by the FP64 pipe,
+// which takes 64 cycles per warp instruction. So no FP64 work is spent on pairs out of
+// range: a row's eight pairs are tested in FP32 with a margin (5e-5 of r_c, far above
+// the rounding of the binary32 positions), and a lane then works off its row's set bits
+// pair by pair with the exact test, taking the next free row of the warp when it has
+// none left. Rows are handed out by ballot ranks once ENVD_REFILL lanes wait: the order
+// depends on the item alone. erfc and its derivative come from one table lookup, and
+// energies share the force's root. The forces of the eight i atoms are kept per lane in
+// shared memory, since a lane's i atom varies. An item is worked off by ENVD_SEG warps,
+// each with a part of its rows. (12 frames of 672 atoms: 1531 us with eight pairs per
+// row and exp and erfc evaluated for the force and for the energy, 301 us; the pipe is
+// 81% busy while a multiprocessor works.)
+__global__ void __launch_bounds__(ENVD_WARPS * 32, 4) k_env_rows_f64(DevPtrs P) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ double s_f[ENVD_WARPS][3 * CL][32];
+    __shared__ Atom<double> s_i[ENVD_WARPS][CL];
+    __shared__ float4 s_p[ENVD_WARPS][CL];
+    __shared__ float4 s_shift[ENVD_WARPS][64];
+    __shared__ int s_item[ENVD_WARPS][8];
+    const KC<double> K = make_kc<double>(P);
+    const float near2 = fmaf(P.rc2, 1e-4f, P.rc2) + 1e-5f;
+    const int n_units = P.ritem_pref[P.R] * ENVD_SEG;
+    const int nw = (int)gridDim.x * ENVD_WARPS;
+    const unsigned int below = (1u << lane) - 1u;
+    volatile int* const I = s_item[w];
+    float4* const sh = s_shift[w];
+    double (*const fl)[32] = s_f[w];
+    int unit = w * (int)gridDim.x + (int)blockIdx.x;
+    while (unit < n_units) {
+        __syncwarp();
+        const RowItem& item = row_item(P, unit / ENVD_SEG);
+        if (lane < 8) I[lane] = reinterpret_cast<const int*>(&item)[lane];
+        __syncwarp();
+        const int rep = P.rep_of_cl[I[0]];
+        const RepDev& R = P.reps[rep];
+        const float4 c = P.xq[I[0] * CL];
+        row_shifts(R, c, lane, sh);
+        if (lane < CL) {
+            const float4 x = P.xq[I[0] * CL + lane];
+            s_p[w][lane] = make_float4(x.x - c.x, x.y - c.y, x.z - c.z, 0.f);
+            Atom<double> ai = load_atom<double>(P, I[0] * CL + lane, R, K);
+            ai.x -= (double)c.x;
+            ai.y -= (double)c.y;
+            ai.z -= (double)c.z;
+            s_i[w][lane] = ai;
+        }
+#pragma unroll
+        for (int q = 0; q < 3 * CL; ++q) fl[q][lane] = 0.0;
+        __syncwarp();
+        const int n = (I[3] & 0xFFFF) + (I[3] >> 16) + I[4] + I[5];
+        const int part = (n + ENVD_SEG - 1) / ENVD_SEG;
+        int next = (unit % ENVD_SEG) * part;
+        const int end = min(n, next + part);
+        unsigned int mask = 0u;   // pairs of this lane's row still to do
+        int ja = 0;
+        Atom<double> a{};
+        T3<double> fj{0.0, 0.0, 0.0};
+        double elj = 0.0, ec = 0.0;
+        for (;;) {
+            const unsigned int need = __ballot_sync(FULL, mask == 0u);
+            if (next < end) {
+                if (__popc(need) >= ENVD_REFILL) {
+                    const int k = next + __popc(need & below);
+                    if (mask == 0u && k < end) {
+                        unsigned int word, em;
+                        env_tail_row(P, I, k, word, em);
+                        ja = (int)(word & ROW_SLOT_MASK);
+                        const int code = (int)(word >> ROW_SLOT_BITS);
+                        const float4 u = sh[code], v = sh[32 + code], x = P.xq[ja];
+                        const float px = (x.x + u.x) - v.x, py = (x.y + u.y) - v.y, pz = (x.z + u.z) - v.z;
+#pragma unroll
+                        for (int ii = 0; ii < CL; ++ii) {
+                            const float4 p = s_p[w][ii];
+                            const float dx = px - p.x, dy = py - p.y, dz = pz - p.z;
+                            mask |= fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < near2 ? 1u << ii : 0u;
+                        }
+                        mask &= ~em;
+                        if (mask) {
+                            a = load_atom<double>(P, ja, R, K);
+                            a.x = ((double)x.x + (double)u.x) - (double)v.x;
+                            a.y = ((double)x.y + (double)u.y) - (double)v.y;
+                            a.z = ((double)x.z + (double)u.z) - (double)v.z;
+                            fj = T3<double>{0.0, 0.0, 0.0};
+                        }
+                    }
+                    next += __popc(need);
+                }
+            } else if (need == FULL) {
+                break;
+            }
+            if (mask) {
+                const int ii = __ffs(mask) - 1;
+                mask &= mask - 1u;
+                const Atom<double> ai = s_i[w][ii];
+                const double dx = a.x - ai.x, dy = a.y - ai.y, dz = a.z - ai.z;
+                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                if (r2 < K.rc2) {
+                    double r, rinv, rinv2, e, d;
+                    root_acc(r2, r, rinv, rinv2);
+                    erfc_table(K.beta * r, K.dtab, e, d);
+                    const double qq = ai.q * a.q;
+                    const double vc = qq * e * rinv;
+                    const double fcr = fma(-(qq * K.beta), d, vc);   // Coulomb force times r^2
+                    const double sig = ai.sh + a.sh;
+                    const double s2 = sig * sig * rinv2;
+                    const double s6 = s2 * s2 * s2;
+                    const double es = ai.e2 * a.e2 * s6;
+                    const double fs = fma(es, fma(12.0, s6, -6.0), fcr) * rinv2;
+                    fl[3 * ii][lane] = fma(-fs, dx, fl[3 * ii][lane]);
+                    fl[3 * ii + 1][lane] = fma(-fs, dy, fl[3 * ii + 1][lane]);
+                    fl[3 * ii + 2][lane] = fma(-fs, dz, fl[3 * ii + 2][lane]);
+                    fj.x = fma(fs, dx, fj.x);
+                    fj.y = fma(fs, dy, fj.y);
+                    fj.z = fma(fs, dz, fj.z);
+                    elj += fma(es, s6, -es);
+                    ec += vc;
+                }
+                if (mask == 0u) {
+                    red_nonzero(P.fx + ja, fj.x);
+                    red_nonzero(P.fy + ja, fj.y);
+                    red_nonzero(P.fz + ja, fj.z);
+                }
+            }
+        }
+        __syncwarp();
+        // i forces: lane v sums value v = 3 ii + c over the warp's lanes
+        if (lane < 3 * CL) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int l = 0; l < 32; ++l) s += fl[lane][(l + lane) & 31];
+            const int cc = lane % 3;
+            red_nonzero((cc == 0 ? P.fx : (cc == 1 ? P.fy : P.fz)) + I[0] * CL + lane / 3, s);
+        }
+        const double sl = warp_sum<double>(elj);
+        const double sc = warp_sum<double>(ec);
+        if (lane == 0) {
+            if (!isfinite(sl) || !isfinite(sc)) set_err(P.cnt, ERRB_NONFINITE, rep);
+            add_fixed(P.eacc + (size_t)rep * EA_N + EA_ENV_LJ, to_fixed_d(sl));
+            add_fixed(P.eacc + (size_t)rep * EA_N + EA_ENV_C, to_fixed_d(sc));
+        }
+        if (nw >= n_units) break;
+        if (lane == 0) unit = nw + atomicAdd(&P.cnt->env_next, 1);
+        unit = __shfl_sync(FULL, unit, 0);
     }
 }
 
@@ -569,9 +718,10 @@ __device__ __forceinline__ void pair_lig(const Atom<T>& ai, const Atom<T>& aj, b
     const T dx = aj.x - ai.x, dy = aj.y - ai.y, dz = aj.z - ai.z;
     const T r2 = fma(dx, dx, fma(dy, dy, dz * dz));
     keep = keep && (r2 < K.rc2);
-    const T r = t_sqrt_acc(r2);
-    const T rinv = t_rcp_acc(r);
-    const T rinv2 = t_rcp_acc(r2);
+    // (FP64: 64 cycles of its pipe per instruction, so a vote pays)
+    if (sizeof(T) == 8 && !__any_sync(FULL, keep)) return;
+    T r, rinv, rinv2;
+    root_acc(r2, r, rinv, rinv2);
     const T qq = ai.q * aj.q;
     T erfcv, ex;
     ewald_acc(r, r2, K, erfcv, ex);
@@ -658,16 +808,17 @@ struct LigEntries {
 
 // Latency bound (a few hundred pairs per window): a warp's first item is its own
 // index (no claim), the entries are loaded together and the j atoms one entry
-// ahead.
+// ahead. In FP64 an item's entries are dealt to LIGD_SEG warps.
 template <typename T, bool ENERGY>
 __global__ void __launch_bounds__(128) k_lig(DevPtrs P) {
     const int lane = threadIdx.x & 31, jj = lane & 7, ii = lane >> 3;
     const KC<T> K = make_kc<T>(P);
-    const int n_items = P.ilig_pref[P.R];
+    constexpr int SEG = sizeof(T) == 8 ? LIGD_SEG : 1;
+    const int n_items = P.ilig_pref[P.R] * SEG;
     const int nw = (int)gridDim.x * 4;
     int it = (threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
     while (it < n_items) {
-        const Item I = P.items_lig[region_index(P.ilig_pref, P.ilig_base, P.R, it)];
+        const Item I = P.items_lig[region_index(P.ilig_pref, P.ilig_base, P.R, it / SEG)];
         const RepDev& R = P.reps[I.rep];
         const int a0 = I.c0 * CL + ii;
         // coordinates relative to the cluster's first atom (see rel_img)
@@ -681,16 +832,17 @@ __global__ void __launch_bounds__(128) k_lig(DevPtrs P) {
         const int ntot = I.e_cnt + I.x_cnt;
         LigEntries L;
         Atom<T> aj_n{};
-        for (int t = 0; t < ntot; ++t) {
-            if ((t & 31) == 0) {
-                L.load(P, I, t, lane);
-                aj_n = load_atom<T>(P, __shfl_sync(FULL, L.e.x, 0) * CL + jj, R, K);
+        for (int t = it % SEG, b = -1; t < ntot; t += SEG) {
+            if ((t & ~31) != b) {
+                b = t & ~31;
+                L.load(P, I, b, lane);
+                aj_n = load_atom<T>(P, __shfl_sync(FULL, L.e.x, t & 31) * CL + jj, R, K);
             }
             const int2 e = make_int2(__shfl_sync(FULL, L.e.x, t & 31), __shfl_sync(FULL, L.e.y, t & 31));
             const unsigned long long m = __shfl_sync(FULL, L.m, t & 31);
             Atom<T> aj = aj_n;
-            if (((t + 1) & 31) != 0 && t + 1 < ntot)
-                aj_n = load_atom<T>(P, __shfl_sync(FULL, L.e.x, (t + 1) & 31) * CL + jj, R, K);
+            if (((t + SEG) & ~31) == b && t + SEG < ntot)
+                aj_n = load_atom<T>(P, __shfl_sync(FULL, L.e.x, (t + SEG) & 31) * CL + jj, R, K);
             const int jlig = entry_jlig(e.y);
             const LigState<T> S = lig_state<T>(P, R, jlig);
             float sx, sy, sz;
@@ -786,8 +938,8 @@ __global__ void __launch_bounds__(UKN_WARPS * 32) k_lig_ukn(DevPtrs P) {
                 const T r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 const bool keep = keep0 && (r2 < K.rc2);
                 if (keep) {
-                    const T r = t_sqrt_acc(r2);
-                    const T rinv = t_rcp_acc(r);
+                    T r, rinv, rinv2;
+                    root_acc(r2, r, rinv, rinv2);
                     T erfcv, ex;
                     ewald_acc(r, r2, K, erfcv, ex);
                     const double u1 = (double)(ai[h].q * aj.q * erfcv * rinv);
@@ -949,24 +1101,24 @@ static bool env_small(const DevPtrs& P, int n_sm) { return P.C <= ENV_SMALL_ITEM
 void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precision, int grid,
                        int block, int n_sm) {
     if (precision == 1) {
-        k_env_rows<double, true, 2><<<grid, block, 0, s>>>(P);
+        k_env_rows_f64<<<grid, ENVD_WARPS * 32, 0, s>>>(P);
     } else if (env_small(P, n_sm)) {
-        if (energy) k_env_rows<float, true, 1><<<grid, block, 0, s>>>(P);
-        else k_env_rows<float, false, 1><<<grid, block, 0, s>>>(P);
+        if (energy) k_env_rows<true, 1><<<grid, block, 0, s>>>(P);
+        else k_env_rows<false, 1><<<grid, block, 0, s>>>(P);
     } else {
-        if (energy) k_env_rows<float, true, 4><<<grid, block, 0, s>>>(P);
-        else k_env_rows<float, false, 4><<<grid, block, 0, s>>>(P);
+        if (energy) k_env_rows<true, 4><<<grid, block, 0, s>>>(P);
+        else k_env_rows<false, 4><<<grid, block, 0, s>>>(P);
     }
 }
 
 int env_kernel_occupancy(int block, int precision, bool energy) {
     int nb = 0;
     if (precision == 1)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<double, true, 2>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows_f64, ENVD_WARPS * 32, 0);
     else if (energy)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, true, 4>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<true, 4>, block, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<float, false, 4>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<false, 4>, block, 0);
     return nb;
 }
 
