@@ -319,7 +319,7 @@ struct DevPtrs {
     const float4* ewtab;           // [EW_NT] Coulomb force table, [EW_NT] erfc(beta r)
     int pme;                       // 1 = reciprocal-space Ewald terms are on
     const double2* pme_self;       // [systems] self energy of the environment / ligand charges
-    const double2* erfc_tab;       // [ERFC_NT][4] erfc's expansions (FP64 contexts)
+    const double2* erfc_tab;       // [ERFC_NT][4] erfc's expansions (FP64 contexts, PME)
     float ewtab_inv_h;             // grid points per unit of r (nm^-1)
     double drc2, dbeta, dke;
     int group, max_entries, ligand_mode;
@@ -366,6 +366,32 @@ __device__ __forceinline__ long long to_fixed_d(double f) {
 }
 __device__ __forceinline__ void add_fixed(long long* p, long long v) {
     atomicAdd(reinterpret_cast<unsigned long long*>(p), static_cast<unsigned long long>(v));
+}
+
+// erfc(x) and its derivative from the expansions about multiples of 1 / 128 (x >= 0;
+// beyond the last point, 8, the value there: 1e-29). Thirteen multiply-adds and two
+// loads' latency where erfc and exp together take over 4,000 issue cycles of the FP64
+// pipe per warp; the remainder is below 1e-16 of the value up to x = 5 and of 1e-13
+// everywhere.
+__device__ __forceinline__ void erfc_table(double x, const double2* tab, double& e, double& d) {
+    const double t = fma(x, (double)ERFC_INV_H, 6755399441055744.0);   // 1.5 * 2^52: rounds to an integer
+    const unsigned int j = min((unsigned int)__double2loint(t), (unsigned int)(ERFC_NT - 1));
+    const double f = fma(t - 6755399441055744.0, -1.0 / ERFC_INV_H, x);
+    const double2* c = tab + (size_t)j * 4;
+    const double2 c67 = c[3], c45 = c[2], c23 = c[1], c01 = c[0];
+    double p = fma(c67.y, f, c67.x);
+    double q = fma(c67.y, f, p);
+    p = fma(p, f, c45.y);
+    q = fma(q, f, p);
+    p = fma(p, f, c45.x);
+    q = fma(q, f, p);
+    p = fma(p, f, c23.y);
+    q = fma(q, f, p);
+    p = fma(p, f, c23.x);
+    q = fma(q, f, p);
+    p = fma(p, f, c01.y);
+    d = fma(q, f, p);
+    e = fma(p, f, c01.x);
 }
 
 // shift of an entry's j cluster, from its packed y word
@@ -476,6 +502,9 @@ struct PmeDev {
     const int* chunks;            // [R+1] prefix of 256-point chunks of the grids
     const int* chunk_rep;         // [n_chunks] replica of each chunk
     int n_chunks;
+    const int* planes;            // [R+1] prefix of xy planes
+    const int* plane_rep;         // [n_planes] replica of each plane
+    int n_planes, plane_elems;    // elements of shared memory that the largest plane needs
     long long total;              // grid points of all replicas
     const double* infl;           // per system: B(m) C(m) at every grid point (0 at m = 0)
     const long long* infl_off;    // [systems]
@@ -490,8 +519,11 @@ struct PmeDev {
 // shared-memory attributes of the FFT kernels, sized for the longest line any
 // context may use (PME_KMAX; a per-process setting), and a check of M.kmax (host only)
 cudaError_t pme_prepare(PmeDev& M);
-void launch_pme_forces(const DevPtrs& P, const PmeDev& M, cudaStream_t s, int n_sm, bool energy);
+// `loaded`: recorded once the transform holds the charges and the charge grid is free
+void launch_pme_forces(const DevPtrs& P, const PmeDev& M, cudaStream_t s, int n_sm, bool energy,
+                       cudaEvent_t loaded);
 void launch_pme_decomposition(const DevPtrs& P, const PmeDev& M, cudaStream_t s, int n_sm);
+void launch_pme_excl(const DevPtrs& P, const PmeDev& M, cudaStream_t s, int n_sm);
 
 // Replica exchange tables. Exchange group = the replicas that share a system and
 // a schedule; within a group, positions 0..n-1 list its replicas by ascending

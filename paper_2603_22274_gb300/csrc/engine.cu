@@ -60,7 +60,7 @@ struct abfe_ctx {
     cudaEvent_t ev_side = nullptr, ev_side2 = nullptr;
     cudaStream_t fork = nullptr;           // ligand pair / bond branch
     cudaStream_t fork2 = nullptr;          // restraint / torsion / PME branch
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr, ev_pme = nullptr;
     int device = 0, n_sm = 0;
     abfe_params prm{};
     abfe_tuning tune{};
@@ -334,9 +334,14 @@ void enqueue_forces(abfe_ctx* c, cudaStream_t s, bool energy, bool fork = true) 
     launch_restraints(c->P, c->pme ? f : f2);
     if (energy) launch_aw_sums(c->P, f2, c->max_aw);
     if (c->pme) {
-        launch_pme_forces(c->P, c->pm, f2, c->n_sm, energy);
-        // energy passes also split the reciprocal energy by charge kind (dU/dlambda_q, u_kn)
-        if (energy) launch_pme_decomposition(c->P, c->pm, f2, c->n_sm);
+        launch_pme_forces(c->P, c->pm, f2, c->n_sm, energy, energy ? c->ev_pme : nullptr);
+        // energy passes also split the reciprocal energy by charge kind (dU/dlambda_q,
+        // u_kn): beside the forces' convolution, once the charge grid is free
+        if (energy) {
+            launch_pme_excl(c->P, c->pm, f, c->n_sm);
+            if (fork) cudaStreamWaitEvent(f, c->ev_pme, 0);
+            launch_pme_decomposition(c->P, c->pm, f, c->n_sm);
+        }
     }
     if (fork) {
         cudaEventRecord(c->ev_join, c->fork);
@@ -520,13 +525,16 @@ abfe_status setup_pme(abfe_ctx* c, const abfe_system_desc* systems, int n_system
     const int R = c->R;
     std::vector<int4> dims(R);
     std::vector<long long> goff(R + 1, 0);
-    std::vector<int> tiles(3 * (R + 1), 0), chunks(R + 1, 0);
+    std::vector<int> tiles(3 * (R + 1), 0), chunks(R + 1, 0), planes(R + 1, 0);
+    c->pm.plane_elems = 0;
     for (int r = 0; r < R; ++r) {
         const int4 K = sdims[c->reps_h[r].sys];
         dims[r] = K;
         const long long pts = (long long)K.x * K.y * K.z;
         goff[r + 1] = goff[r] + pts;
         chunks[r + 1] = chunks[r] + (int)((pts + 255) / 256);
+        planes[r + 1] = planes[r] + K.z;
+        c->pm.plane_elems = std::max(c->pm.plane_elems, 2 * K.y * (K.x | 1) + K.x + K.y);
         const int Ka[3] = {K.x, K.y, K.z};
         for (int a = 0; a < 3; ++a) {
             const int b = a == 0 ? 1 : 0, cc = a == 2 ? 1 : 2;
@@ -559,11 +567,16 @@ abfe_status setup_pme(abfe_ctx* c, const abfe_system_desc* systems, int n_system
         for (int r = 0; r < R; ++r)
             for (int t = tiles[a * (R + 1) + r]; t < tiles[a * (R + 1) + r + 1]; ++t) tile_rep[a][t] = r;
     }
-    for (int r = 0; r < R; ++r)
+    std::vector<int> plane_rep(planes[R]);
+    for (int r = 0; r < R; ++r) {
         for (int t = chunks[r]; t < chunks[r + 1]; ++t) chunk_rep[t] = r;
+        for (int t = planes[r]; t < planes[r + 1]; ++t) plane_rep[t] = r;
+    }
     int* d_tile_rep[3];
     for (int a = 0; a < 3; ++a) d_tile_rep[a] = dalloc<int>(c, tile_rep[a].size(), ok);
     int* d_chunk_rep = dalloc<int>(c, chunk_rep.size(), ok);
+    int* d_planes = dalloc<int>(c, R + 1, ok);
+    int* d_plane_rep = dalloc<int>(c, plane_rep.size(), ok);
     double* d_infl = dalloc<double>(c, infl.size(), ok);
     long long* d_infl_off = dalloc<long long>(c, n_systems, ok);
     double2* d_twd = dalloc<double2>(c, twd.size(), ok);
@@ -584,6 +597,8 @@ abfe_status setup_pme(abfe_ctx* c, const abfe_system_desc* systems, int n_system
     up(d_chunks, chunks.data(), sizeof(int) * (R + 1));
     for (int a = 0; a < 3; ++a) up(d_tile_rep[a], tile_rep[a].data(), sizeof(int) * tile_rep[a].size());
     up(d_chunk_rep, chunk_rep.data(), sizeof(int) * chunk_rep.size());
+    up(d_planes, planes.data(), sizeof(int) * (R + 1));
+    up(d_plane_rep, plane_rep.data(), sizeof(int) * plane_rep.size());
     up(d_infl, infl.data(), sizeof(double) * infl.size());
     up(d_infl_off, infl_off.data(), sizeof(long long) * n_systems);
     up(d_twd, twd.data(), sizeof(double2) * twd.size());
@@ -603,6 +618,9 @@ abfe_status setup_pme(abfe_ctx* c, const abfe_system_desc* systems, int n_system
     }
     M.chunks = d_chunks;
     M.chunk_rep = d_chunk_rep;
+    M.planes = d_planes;
+    M.plane_rep = d_plane_rep;
+    M.n_planes = planes[R];
     for (int a = 0; a < 3; ++a) M.tile_rep[a] = d_tile_rep[a];
     M.infl = d_infl;
     M.infl_off = d_infl_off;
@@ -851,6 +869,7 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
     cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
     cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
     cudaEventCreateWithFlags(&c->ev_join2, cudaEventDisableTiming);
+    cudaEventCreateWithFlags(&c->ev_pme, cudaEventDisableTiming);
     c->tune.group = p->precision == 1 ? 1 : 2;
     c->tune.max_entries = 64;
     c->tune.block_threads = 128;
@@ -1289,7 +1308,7 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
             return set_error(nullptr, ABFE_ERR_OUT_OF_MEMORY, "Ewald table");
         }
         P.ewtab = d_tab;
-        if (p->precision == 1) {
+        if (p->precision == 1 || p->pme_order > 0) {
             // erfc's Taylor coefficients from those of g = exp(-x^2), whose derivative
             // is -2 x g: (n + 1) g_{n+1} = -2 (x_j g_n + g_{n-1})
             std::vector<double> et((size_t)ERFC_NT * 8);
@@ -1444,6 +1463,7 @@ void abfe_destroy(abfe_ctx* c) {
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->ev_join2) cudaEventDestroy(c->ev_join2);
+    if (c->ev_pme) cudaEventDestroy(c->ev_pme);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
 }

@@ -88,32 +88,6 @@ __device__ __forceinline__ Atom<double> load_atom<double>(const DevPtrs& P, int 
 }
 
 
-// erfc(x) and its derivative from the expansions about multiples of 1 / 128 (x >= 0;
-// beyond the last point, 8, the value there: 1e-29). Thirteen multiply-adds and two
-// loads' latency where erfc and exp together take over 4,000 issue cycles of the FP64
-// pipe per warp; the remainder is below 1e-16 of the value up to x = 5 and of 1e-13
-// everywhere.
-__device__ __forceinline__ void erfc_table(double x, const double2* tab, double& e, double& d) {
-    const double t = fma(x, (double)ERFC_INV_H, 6755399441055744.0);   // 1.5 * 2^52: rounds to an integer
-    const unsigned int j = min((unsigned int)__double2loint(t), (unsigned int)(ERFC_NT - 1));
-    const double f = fma(t - 6755399441055744.0, -1.0 / ERFC_INV_H, x);
-    const double2* c = tab + (size_t)j * 4;
-    const double2 c67 = c[3], c45 = c[2], c23 = c[1], c01 = c[0];
-    double p = fma(c67.y, f, c67.x);
-    double q = fma(c67.y, f, p);
-    p = fma(p, f, c45.y);
-    q = fma(q, f, p);
-    p = fma(p, f, c45.x);
-    q = fma(q, f, p);
-    p = fma(p, f, c23.y);
-    q = fma(q, f, p);
-    p = fma(p, f, c23.x);
-    q = fma(q, f, p);
-    p = fma(p, f, c01.y);
-    d = fma(q, f, p);
-    e = fma(p, f, c01.x);
-}
-
 // G(r) from the shared-memory table: the nearest grid point j = round(t),
 // t = r / h (clamped to the table), and the centred quadratic in f = t - j.
 // Adding 1.5 * 2^23 leaves round(t) in the low mantissa bits (t < 2^22), so no
