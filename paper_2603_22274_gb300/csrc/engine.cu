@@ -74,7 +74,7 @@ struct abfe_ctx {
     std::vector<int> rep_of_cl_h;
     std::vector<int64_t> rep_atom_off;
     int64_t total_atoms = 0;
-    int S = 0, C = 0, NCOL = 0, max_bonds = 0, n_lig_cl = 0, max_lig_cl = 0;
+    int S = 0, C = 0, NCOL = 0, max_bonds = 0, n_lig_cl = 0, max_lig_cl = 0, max_cl_cap = 0;
     int n_bond_total = 0;
     int64_t epc_max = 0;                   // outer entries per cluster, the largest estimate
     int max_aw = 0;
@@ -332,7 +332,7 @@ void enqueue_forces(abfe_ctx* c, cudaStream_t s, bool energy, bool fork = true) 
     if (fork) prof_rec(c, c->ev_lig, false, f);
     launch_bonds(c->P, f, c->prm.precision, energy);
     launch_restraints(c->P, c->pme ? f : f2);
-    if (energy) launch_aw_sums(c->P, f2, c->max_aw);
+    if (energy) launch_aw_sums(c->P, f2, c->max_aw, c->max_cl_cap);
     if (c->pme) {
         launch_pme_forces(c->P, c->pm, f2, c->n_sm, energy, energy ? c->ev_pme : nullptr);
         // energy passes also split the reciprocal energy by charge kind (dU/dlambda_q,
@@ -1031,6 +1031,7 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         const int nlc = (nl + CL - 1) / CL;
         c->n_lig_cl += nlc;
         c->max_lig_cl = std::max(c->max_lig_cl, nlc);
+        c->max_cl_cap = std::max(c->max_cl_cap, R.n_cl_cap);
         // A ligand cluster's list is a full list (no half-list rule) and its
         // bounding box is as long as its stretch of the chain, so no density
         // estimate bounds it: size the ligand items for every cluster of the
