@@ -442,8 +442,9 @@ abfe_status abfe_ukn_frame_noalloc(const abfe_noalloc_frame *frame, double *d_du
  *    ABFE_ERR_NONFINITE (a non-finite u_kn or free energy); ABFE_ERR_OUT_OF_MEMORY;
  *    ABFE_ERR_CUDA. The message is abfe_last_error(NULL).
  *  - Device scratch of about 8 (K N + N + 2 K N / 16384 + K min(N / 32, twice
- *    the SM count) + 5 K) bytes, plus 8 K N bytes for the copy of u_kn in abfe_mbar, comes from the allocator
- *    installed by abfe_set_allocator (else cudaMalloc) and is freed on return.
+ *    the SM count) + 5 K) bytes, plus 8 K N bytes for the copy of u_kn in
+ *    abfe_mbar, comes from the allocator installed by abfe_set_allocator (else
+ *    cudaMalloc) and is freed on return.
  */
 #define ABFE_MBAR_MAX_K 1024
 abfe_status abfe_mbar(const double *h_u_kn, const int32_t *h_N_k, int32_t K, int64_t N,

@@ -201,6 +201,7 @@ struct Counters {
     unsigned long long n_win_rebuilds, n_win_prunes;   // windows rebuilt / pruned, summed
     unsigned long long ex_attempt; // replica-exchange attempts so far (the RNG counter)
     long long ex_accepted;         // accepted swaps so far
+    int bad_input;      // the coordinates or velocities just staged hold a non-finite value
 };
 
 struct StepParams {
@@ -486,6 +487,8 @@ void launch_finalize(const DevPtrs& P, cudaStream_t s);
 void launch_ukn_assemble(const DevPtrs& P, cudaStream_t s, double kT);
 void launch_scatter_out(const DevPtrs& P, cudaStream_t s, int what, double* outd, float* outf,
                         int n_sm);
+// flags a non-finite value among n staged doubles; launch_gather_in then leaves the state as it is
+void launch_check_in(const DevPtrs& P, cudaStream_t s, const double* in, int64_t n, int n_sm);
 void launch_gather_in(const DevPtrs& P, cudaStream_t s, int what, const double* in, int n_sm);
 
 // Smooth-PME grids of all replicas (see pme.cu).

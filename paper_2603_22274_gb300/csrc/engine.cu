@@ -383,11 +383,18 @@ void enqueue_prepare(abfe_ctx* c, cudaStream_t s) {
     c->force_prune = false;
 }
 
-abfe_status check_device(abfe_ctx* c) {
+// bad_input: set when staged input was refused (see k_check_in)
+abfe_status check_device(abfe_ctx* c, bool* bad_input = nullptr) {
     CK(cudaStreamSynchronize(c->stream));
     CK(cudaGetLastError());
     Counters h;
     CK(cudaMemcpy(&h, c->d_cnt, sizeof(Counters), cudaMemcpyDeviceToHost));
+    if (h.bad_input) {
+        const int none = 0;
+        CK(cudaMemcpy(&c->d_cnt->bad_input, &none, sizeof(int), cudaMemcpyHostToDevice));
+        if (bad_input) *bad_input = true;
+        return set_error(c, ABFE_ERR_NONFINITE, "non-finite input");
+    }
     if (h.err == 0) return ABFE_OK;
     int zero = 0;
     CK(cudaMemcpy(&c->d_cnt->err, &zero, sizeof(int), cudaMemcpyHostToDevice));
@@ -2050,15 +2057,16 @@ static abfe_status io_atoms(abfe_ctx* c, int what, double* out, const double* in
     }
     const size_t bytes = sizeof(double) * 3 * c->total_atoms;
     if (in) {
-        if (!finite3(in, 3 * c->total_atoms)) return set_error(c, ABFE_ERR_NONFINITE, "non-finite input");
         CK(cudaMemcpyAsync(c->d_atom3, in, bytes, cudaMemcpyHostToDevice, c->stream));
+        launch_check_in(c->P, c->stream, c->d_atom3, 3 * c->total_atoms, c->n_sm);
         launch_gather_in(c->P, c->stream, what, c->d_atom3, c->n_sm);
-        if (what == 2) {
+        bool bad = false;
+        const abfe_status st = check_device(c, &bad);
+        if (what == 2 && !bad) {
             c->force_rebuild = true;
             c->f_valid = false;
         }
-        CK(cudaStreamSynchronize(c->stream));
-        return check_device(c);
+        return st;
     }
     launch_scatter_out(c->P, c->stream, what, c->d_atom3, nullptr, c->n_sm);
     CK(cudaStreamSynchronize(c->stream));
