@@ -117,6 +117,12 @@ struct abfe_ctx {
     std::string err;
     int env_grid = 0, lig_grid = 0;
     cudaGraphExec_t gexec = nullptr;
+    // the unforced list decision of a force pass (see prepare_graph), the parameters that
+    // it was captured with, how many such passes ran, and whether its capture failed
+    cudaGraphExec_t prep = nullptr;
+    DevPtrs prep_P;
+    int prep_calls = 0;
+    bool prep_failed = false;
     int g_steps = 0;
     bool g_prof = false;
     int g_mode = 0;  // 1 = conditional rebuild node, 2 = predicated rebuild kernels
@@ -225,6 +231,7 @@ abfe_status ensure_rows(abfe_ctx* c, double prune_skin) {
 
 void free_all(abfe_ctx* c) {
     if (c->gexec) { cudaGraphExecDestroy(c->gexec); c->gexec = nullptr; }
+    if (c->prep) { cudaGraphExecDestroy(c->prep); c->prep = nullptr; }
     cudaStreamSynchronize(c->stream);
     for (auto& a : c->allocs) {
         if (g_free) g_free(a.first, a.second, (void*)c->stream, g_user);
@@ -365,9 +372,16 @@ StepEnd forced_end(bool rebuild, bool prune) {
     return e;
 }
 
+bool prepare_graph(abfe_ctx* c);
+
 // zero forces, displacement check, rebuild and prune decisions, (predicated)
 // outer rebuild and prune
 void enqueue_prepare(abfe_ctx* c, cudaStream_t s) {
+    if (!c->force_rebuild && !c->force_prune && s == c->stream && prepare_graph(c)) {
+        if (cudaGraphLaunch(c->prep, s) == cudaSuccess) return;
+        cudaGetLastError();
+        c->prep_failed = true;
+    }
     launch_integrate(with_sp(c, SP_ZERO), s, c->n_sm, forced_end(c->force_rebuild, c->force_prune));
     // host-forced builds and prunes are timed while profiling is on
     const bool tb = c->force_rebuild, tp = c->force_rebuild || c->force_prune;
@@ -1766,6 +1780,56 @@ static bool capture_cond(abfe_ctx* c, cudaStream_t s, cudaGraphConditionalHandle
     return cudaStreamUpdateCaptureDependencies(s, &cn, nullptr, 1,
                                                cudaStreamSetCaptureDependencies) == cudaSuccess;
 }
+
+namespace {
+
+// A force pass that forces no list update needs the decision (the integrator's last
+// block) and, mostly, none of the ten list kernels behind it: as a graph with one
+// conditional node it is one launch of the host's instead of eleven, which bounded small
+// frames (one 4,500-atom window: 83 -> 64 us a pass). Captured at the PREP_CALLS-th
+// such pass, so that a context that makes few of them does not pay for it, and again when
+// a parameter of the kernels changed. False: not captured (yet).
+constexpr int PREP_CALLS = 8;
+bool prepare_graph(abfe_ctx* c) {
+    if (c->prep && std::memcmp(&c->prep_P, &c->P, sizeof(DevPtrs)) == 0) return true;
+    if (c->prep_failed || ++c->prep_calls < PREP_CALLS) return false;
+    if (c->prep) cudaGraphExecDestroy(c->prep);
+    c->prep = nullptr;
+    c->prep_calls = 0;
+    cudaGraph_t g = nullptr;
+    bool ok = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        StepEnd end = forced_end(false, false);
+        cudaStreamCaptureStatus cs;
+        unsigned long long id;
+        cudaGraph_t cap;
+        end.use_handle = 1;
+        ok = cudaStreamGetCaptureInfo(c->stream, &cs, &id, &cap, nullptr, nullptr, nullptr) == cudaSuccess &&
+             cudaGraphConditionalHandleCreate(&end.h_update, cap, 2, 0) == cudaSuccess;
+        if (ok) {
+            launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm, end);
+            ok = capture_cond(c, c->stream, end.h_update,
+                              {[&](cudaStream_t b) { launch_prune(c->P, b, c->n_sm); }, [&](cudaStream_t b) {
+                                   launch_rebuild(c->P, b, c->n_sm);
+                                   launch_list_build(c->P, b, c->max_lig_cl, c->side2, c->ev_side, c->ev_side2);
+                                   launch_prune(c->P, b, c->n_sm);
+                               }});
+        }
+        const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+        ok = ok && e == cudaSuccess && g && cudaGraphInstantiate(&c->prep, g, 0) == cudaSuccess;
+        if (g) cudaGraphDestroy(g);
+    }
+    if (!ok) {
+        cudaGetLastError();
+        c->prep = nullptr;
+        c->prep_failed = true;
+        return false;
+    }
+    std::memcpy(&c->prep_P, &c->P, sizeof(DevPtrs));
+    return true;
+}
+
+}  // namespace
 
 extern "C" {
 
