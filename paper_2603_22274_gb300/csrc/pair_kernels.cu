@@ -9,8 +9,9 @@
 //   force goes to the 64-bit fixed-point accumulators once per row and the i
 //   forces stay in registers until the item ends. FP32 forces: the Coulomb force is
 //   qq G(r) / r^3 with G from a quadratic table in r held in shared memory
-//   (ewald_G); FP32 energies (energy steps only) use correctly rounded
-//   arithmetic and erfcf/expf; FP64 uses erfc/exp.
+//   (ewald_G); FP32 energies (energy steps only) use erfc from a second table and
+//   the force's reciprocal root, corrected.
+// * k_env_rows_f64: the same pairs in FP64 contexts, erfc from Taylor coefficients.
 // * k_lig: ligand-involved pairs at the replica's own state (outer list, 4x8
 //   half tiles: lane = jj + 8 ii): Beutler softcore LJ, lambda_q-scaled
 //   charges, dU/dlambda_v and dU/dlambda_q; pair arithmetic in the kernel's
@@ -114,8 +115,8 @@ __device__ __forceinline__ float ewald_erfc(float r, const float4* tab, float in
     return c.x + fmaf(fmaf(c.z, f, c.y), f, c.w);
 }
 
-// correctly rounded / library-accurate variants, used where energies are
-// summed for dU/dlambda and u_kn (ligand pairs, energy steps)
+// correctly rounded / library-accurate variants, used for ligand pairs (dU/dlambda and
+// u_kn)
 __device__ __forceinline__ float t_sqrt_acc(float x) { return __fsqrt_rn(x); }
 __device__ __forceinline__ float t_rcp_acc(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double t_rcp_acc(double x) { return 1.0 / x; }
