@@ -473,8 +473,11 @@ void launch_lig_ukn(const DevPtrs& P, cudaStream_t s, int grid, int precision);
 void launch_count_pairs(const DevPtrs& P, cudaStream_t s, int grid, int block);
 // what the integrator's last block does after it (on = 0: nothing): count the
 // step, decide on rebuilds and prunes (forced ones too), set the graph conditionals
+// that the capture around it created (a force pass's graph has no exchange node,
+// whether exchanges are on in the context or not)
 struct StepEnd {
-    int on = 0, inc_step = 0, force_rebuild = 0, force_prune = 0, use_handle = 0;
+    int on = 0, inc_step = 0, force_rebuild = 0, force_prune = 0;
+    int has_update = 0, has_exchange = 0;   // the handles below exist
     cudaGraphConditionalHandle h_update = 0, h_exchange = 0;
 };
 void launch_integrate(const DevPtrs& P, cudaStream_t s, int n_sm, const StepEnd& end = StepEnd{});

@@ -1803,7 +1803,7 @@ bool prepare_graph(abfe_ctx* c) {
         cudaStreamCaptureStatus cs;
         unsigned long long id;
         cudaGraph_t cap;
-        end.use_handle = 1;
+        end.has_update = 1;
         ok = cudaStreamGetCaptureInfo(c->stream, &cs, &id, &cap, nullptr, nullptr, nullptr) == cudaSuccess &&
              cudaGraphConditionalHandleCreate(&end.h_update, cap, 2, 0) == cudaSuccess;
         if (ok) {
@@ -1845,9 +1845,10 @@ static bool enqueue_step(abfe_ctx* c, cudaStream_t s, int mode) {
         cudaGraph_t g;
         if (cudaStreamGetCaptureInfo(s, &cs, &id, &g, nullptr, nullptr, nullptr) != cudaSuccess)
             return false;
-        end.use_handle = 1;
+        end.has_update = 1;
         if (cudaGraphConditionalHandleCreate(&end.h_update, g, 2, 0) != cudaSuccess) return false;
-        if (c->ex_every > 0 &&
+        end.has_exchange = c->ex_every > 0 ? 1 : 0;
+        if (end.has_exchange &&
             cudaGraphConditionalHandleCreate(&end.h_exchange, g, 0, 0) != cudaSuccess)
             return false;
     } else if (mode == 2 && c->ex_every > 0) {

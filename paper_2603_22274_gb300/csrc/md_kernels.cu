@@ -159,13 +159,11 @@ __device__ __forceinline__ void step_end(const DevPtrs& P, const StepEnd& E) {
         }
         s_rb = rb;
         s_pr = pr;
-        if (E.use_handle) {
-            // bodies of the update node: 0 prune, 1 rebuild and prune, else nothing
-            cudaGraphSetConditional(E.h_update, rb ? 1u : (pr ? 0u : 2u));
-            // a replica-exchange attempt ends every ex_every-th step
-            if (P.ex_every > 0)
-                cudaGraphSetConditional(E.h_exchange, (step % (unsigned long long)P.ex_every) == 0ull ? 1u : 0u);
-        }
+        // bodies of the update node: 0 prune, 1 rebuild and prune, else nothing
+        if (E.has_update) cudaGraphSetConditional(E.h_update, rb ? 1u : (pr ? 0u : 2u));
+        // a replica-exchange attempt ends every ex_every-th step
+        if (E.has_exchange)
+            cudaGraphSetConditional(E.h_exchange, (step % (unsigned long long)P.ex_every) == 0ull ? 1u : 0u);
     }
     __syncthreads();
     // per replica: rebuilt in this step when any of its atoms left its half of
