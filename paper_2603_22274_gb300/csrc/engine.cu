@@ -1788,34 +1788,43 @@ namespace {
 // conditional node it is one launch of the host's instead of eleven, which bounded small
 // frames (one 4,500-atom window: 83 -> 64 us a pass). Captured at the PREP_CALLS-th
 // such pass, so that a context that makes few of them does not pay for it, and again when
-// a parameter of the kernels changed. False: not captured (yet).
+// a parameter of the kernels changed. The capture runs on a stream of the context's own:
+// on the caller's it would take in what other threads put there meanwhile, and the legacy
+// default stream cannot be captured. A caller who is capturing the stream gets the direct
+// launches. False: no graph to launch.
 constexpr int PREP_CALLS = 8;
 bool prepare_graph(abfe_ctx* c) {
+    if (c->prep_failed) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
     if (c->prep && std::memcmp(&c->prep_P, &c->P, sizeof(DevPtrs)) == 0) return true;
-    if (c->prep_failed || ++c->prep_calls < PREP_CALLS) return false;
+    if (++c->prep_calls < PREP_CALLS) return false;
     if (c->prep) cudaGraphExecDestroy(c->prep);
     c->prep = nullptr;
     c->prep_calls = 0;
+    cudaStream_t s = c->fork;   // capture_cond records the bodies on `side` and `side2`
     cudaGraph_t g = nullptr;
-    bool ok = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    bool ok = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
         StepEnd end = forced_end(false, false);
-        cudaStreamCaptureStatus cs;
         unsigned long long id;
-        cudaGraph_t cap;
+        cudaGraph_t cg;
         end.has_update = 1;
-        ok = cudaStreamGetCaptureInfo(c->stream, &cs, &id, &cap, nullptr, nullptr, nullptr) == cudaSuccess &&
-             cudaGraphConditionalHandleCreate(&end.h_update, cap, 2, 0) == cudaSuccess;
+        ok = cudaStreamGetCaptureInfo(s, &cap, &id, &cg, nullptr, nullptr, nullptr) == cudaSuccess &&
+             cudaGraphConditionalHandleCreate(&end.h_update, cg, 2, 0) == cudaSuccess;
         if (ok) {
-            launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm, end);
-            ok = capture_cond(c, c->stream, end.h_update,
+            launch_integrate(with_sp(c, SP_ZERO), s, c->n_sm, end);
+            ok = capture_cond(c, s, end.h_update,
                               {[&](cudaStream_t b) { launch_prune(c->P, b, c->n_sm); }, [&](cudaStream_t b) {
                                    launch_rebuild(c->P, b, c->n_sm);
                                    launch_list_build(c->P, b, c->max_lig_cl, c->side2, c->ev_side, c->ev_side2);
                                    launch_prune(c->P, b, c->n_sm);
                                }});
         }
-        const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+        const cudaError_t e = cudaStreamEndCapture(s, &g);
         ok = ok && e == cudaSuccess && g && cudaGraphInstantiate(&c->prep, g, 0) == cudaSuccess;
         if (g) cudaGraphDestroy(g);
     }
