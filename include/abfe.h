@@ -195,10 +195,11 @@ typedef struct {
     int64_t steps_done;
     int64_t slots, clusters;              /* padded atom slots and clusters (all replicas) */
     int64_t device_bytes;                 /* device memory held by the context */
-    int64_t env_lane_groups;              /* pair lanes the environment kernel computes over
-                                             the inner list, divided by 32 (a warp round of
-                                             32 rows counts 4 for each half block of i atoms
-                                             it evaluates), from the last abfe_count_pairs */
+    int64_t env_lane_groups;              /* pair lanes the FP32 environment kernel computes over
+                                             the inner list, divided by 32: 8 for every round
+                                             of up to 32 rows of a work item (all 8 i atoms,
+                                             half rows included), from the last
+                                             abfe_count_pairs */
     int64_t n_prunes;                     /* inner-list prune events (any window) since create */
     int64_t n_rows, n_xrows;              /* inner-list rows (plain, with excluded pairs) */
     int64_t n_exchange_attempts;          /* abfe_replica_exchange calls since create (or as

@@ -4,10 +4,11 @@
 //   12-6 LJ with Lorentz-Berthelot mixing plus real-space Ewald Coulomb, hard
 //   cutoff, over the inner list of j rows. A warp owns one i-cluster (8 atoms,
 //   held in shared memory) and walks its rows 32 at a time, a lane per row:
-//   the lane loads the row's j atom once and evaluates it against the i atoms
-//   the row covers (all 8 of a full row; atoms 0-3 or 4-7 of a half row); its j
-//   force goes to the 64-bit fixed-point accumulators once per row and the i
-//   forces stay in registers until the item ends. FP32 forces: the Coulomb force is
+//   the lane loads the row's j atom once and evaluates it against all 8 i atoms,
+//   dropping those that the row does not cover (atoms 4-7 or 0-3 of a half row,
+//   excluded ones of a masked row); its j force goes to the 64-bit fixed-point
+//   accumulators once per row and the i forces stay in registers until the item
+//   ends. FP32 forces: the Coulomb force is
 //   qq G(r) / r^3 with G from a quadratic table in r held in shared memory
 //   (ewald_G); FP32 energies (energy steps only) use erfc from a second table and
 //   the force's reciprocal root, corrected.
@@ -953,11 +954,11 @@ __global__ void __launch_bounds__(UKN_WARPS * 32) k_lig_ukn(DevPtrs P) {
 }
 
 // ------------------------------------------------------------------ pair counting
-// Environment pairs through the inner rows (the list the force kernel walks),
-// in the force kernel's lane layout (lane per row, 32 rows per round, plain
-// then masked rows); the item's computed pairs go to pair_cnt[2 R] in units
-// of 32 for the lane efficiency: per round 32 lanes x 4 for each half block
-// (atoms 0-3, 4-7) that some row of the round needs.
+// Environment pairs through the inner rows (the list the force kernel walks), in the
+// FP32 force kernel's lane layout (lane per row, 32 rows per round, plain then masked
+// rows); the pairs that kernel evaluates for the item go to pair_cnt[2 R] in units of
+// 32, for the lane efficiency: all eight i atoms for each lane of every round, half rows
+// and the idle lanes of the last round included.
 __global__ void __launch_bounds__(128) k_count_rows(DevPtrs P) {
     const int lane = threadIdx.x & 31;
     const int n_items = P.ritem_pref[P.R];
@@ -967,7 +968,6 @@ __global__ void __launch_bounds__(128) k_count_rows(DevPtrs P) {
         const int rep = P.rep_of_cl[I.c];
         const RepDev& R = P.reps[rep];
         int cnt = 0;
-        long long lanes = 0;
         const int n_full = I.cnt & 0xFFFF, n_lo_end = n_full + I.n_lo;
         const int n_plain = n_lo_end + I.n_hi, n = n_plain + (I.cnt >> 16);
         for (int k0 = 0; k0 < n; k0 += 32) {
@@ -975,8 +975,6 @@ __global__ void __launch_bounds__(128) k_count_rows(DevPtrs P) {
             const bool valid = k < n, masked = k >= n_plain;
             const bool act_lo = valid && (masked || k < n_lo_end);
             const bool act_hi = valid && (masked || k < n_full || k >= n_lo_end);
-            lanes += 128LL * ((__any_sync(0xffffffffu, act_lo) ? 1 : 0) +
-                              (__any_sync(0xffffffffu, act_hi) ? 1 : 0));
             if (!valid) continue;
             unsigned int word, em = 0u;
             if (masked) {
@@ -1011,9 +1009,9 @@ __global__ void __launch_bounds__(128) k_count_rows(DevPtrs P) {
         if (lane == 0 && tot)
             atomicAdd(reinterpret_cast<unsigned long long*>(P.pair_cnt + (size_t)rep * 2),
                       (unsigned long long)tot);
-        if (lane == 0 && lanes)
+        if (lane == 0)
             atomicAdd(reinterpret_cast<unsigned long long*>(P.pair_cnt + (size_t)P.R * 2),
-                      (unsigned long long)(lanes / 32));
+                      (unsigned long long)(CL * ((n + 31) / 32)));
     }
 }
 
