@@ -209,31 +209,32 @@ __device__ void mbar_linear(const MbarDev& M, double* sm) {
         __syncthreads();
         if (tid < tn) s_d[tid] = inv;
         __syncthreads();
-        const int m0 = cnt * s_of / seg, m1 = cnt * (s_of + 1) / seg;
-        if (s_of < seg) {
+        // the longest segment's trip count and whole warps for all lanes (segments change
+        // within a warp and some lanes have none), so that the votes take full warps
+        const int m0 = cnt * s_of / seg, m1 = cnt * (s_of + 1) / seg, len = (cnt + seg - 1) / seg;
 #pragma unroll
-            for (int q = 0; q < MB_SUMS; ++q) {
-                const int i = i_of + q * MB_THREADS;
-                if (i >= K) break;
-                const double* row = s_c + (size_t)i * ls;
-                double s[4] = {0.0, 0.0, 0.0, 0.0};
-                for (int m = m0; m < m1; m += 4) {
-                    double v[4], r[4];
-                    bool nz = false;
+        for (int q = 0; q < MB_SUMS; ++q) {
+            if (q * MB_THREADS >= K) break;
+            const int i = i_of + q * MB_THREADS;
+            const int end = s_of < seg && i < K ? m1 : 0;
+            const double* row = s_c + (size_t)i * ls;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int m = m0; m < m0 + len; m += 4) {
+                double v[4], r[4];
+                bool nz = false;
 #pragma unroll
-                    for (int p = 0; p < 4; ++p) {
-                        const bool on = m + p < m1;
-                        v[p] = on ? row[m + p] : 0.0;
-                        r[p] = on ? s_d[m + p] : 0.0;
-                        nz |= __double_as_longlong(v[p]) != 0ll;
-                    }
-                    if (__any_sync(__activemask(), nz)) {
-#pragma unroll
-                        for (int p = 0; p < 4; ++p) s[p] = fma(v[p], r[p], s[p]);
-                    }
+                for (int p = 0; p < 4; ++p) {
+                    const bool on = m + p < end;
+                    v[p] = on ? row[m + p] : 0.0;
+                    r[p] = on ? s_d[m + p] : 0.0;
+                    nz |= __double_as_longlong(v[p]) != 0ll;
                 }
-                sum[q] += (s[0] + s[1]) + (s[2] + s[3]);
+                if (__any_sync(0xffffffffu, nz)) {
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) s[p] = fma(v[p], r[p], s[p]);
+                }
             }
+            sum[q] += (s[0] + s[1]) + (s[2] + s[3]);
         }
     }
     // the segments of a state, in order
