@@ -49,11 +49,11 @@ constexpr int EW_NT = 1024;
 // FP64 expansions of erfc(x) about x = j / ERFC_INV_H, j < ERFC_NT: eight Taylor
 // coefficients each (up to (x - x_j)^7)
 constexpr int ERFC_NT = 1025, ERFC_INV_H = 128;
-// FP64 pair kernels: warps per block and per item of the row kernel, idle lanes that
-// make it refill, warps per item of the ligand kernel (12 frames of 672 atoms: row
-// kernel's 1, 2, 4, 8 per item 501, 476, 550, 608 us a pass; refills at 4, 8, 12 idle
-// lanes 502, 502, 511; ligand kernel's 1, 2, 4 per item 476, 458, 457)
-constexpr int ENVD_WARPS = 4, ENVD_SEG = 2, ENVD_REFILL = 8, LIGD_SEG = 2;
+// FP64 pair kernels: warps per item of the row kernel, idle lanes that make it refill,
+// warps per item of the ligand kernel (12 frames of 672 atoms: row kernel's 1, 2, 4, 8
+// per item 501, 476, 550, 608 us a pass; refills at 4, 8, 12 idle lanes 502, 502, 511;
+// ligand kernel's 1, 2, 4 per item 476, 458, 457)
+constexpr int ENVD_SEG = 2, ENVD_REFILL = 8, LIGD_SEG = 2;
 constexpr int COL_MAX = 1024;       // atoms per column (per-column sort capacity)
 constexpr double FSCALE = 4294967296.0;
 constexpr float FSCALEF = 4294967296.0f;
@@ -466,6 +466,8 @@ void launch_list_build(const DevPtrs& P, cudaStream_t s, int max_lig_cl, cudaStr
 void launch_prune(const DevPtrs& P, cudaStream_t s, int n_sm);
 void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precision, int grid,
                        int block, int n_sm);
+// shared-memory attribute of the FP64 row kernel, for the largest block of any tuning
+cudaError_t env_prepare();
 int env_kernel_occupancy(int block, int precision, bool energy);
 void launch_lig_forces(const DevPtrs& P, cudaStream_t s, int precision, int grid, int block,
                        bool energy);

@@ -665,7 +665,7 @@ void update_grids(abfe_ctx* c) {
     // from the kernels beside them (one solvent window: 53 us of pair kernel next to
     // its forked neighbours, 37 alone)
     const bool f64 = c->prm.precision == 1;
-    const int warps = f64 ? ENVD_WARPS : c->tune.block_threads / 32;
+    const int warps = c->tune.block_threads / 32;
     const int64_t items = (int64_t)c->C * (1 + c->epc_max / c->tune.max_entries) * (f64 ? ENVD_SEG : 1);
     c->env_grid = (int)std::min<int64_t>((int64_t)c->n_sm * occ,
                                          std::max<int64_t>(c->n_sm, (items + warps - 1) / warps));
@@ -1360,6 +1360,11 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
     P.dbeta = p->ewald_beta;
     P.dke = p->coulomb_k;
     P.ligand_mode = p->ligand_mode;
+    if (p->precision == 1 && env_prepare() != cudaSuccess) {
+        cudaGetLastError();
+        abfe_destroy(c);
+        return set_error(nullptr, ABFE_ERR_CUDA, "FP64 pair kernel attributes");
+    }
     update_grids(c);
 
     // ---------------------------------------------------------------- uploads

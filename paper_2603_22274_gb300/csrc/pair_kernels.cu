@@ -546,21 +546,26 @@ __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
 // each with a part of its rows. (12 frames of 672 atoms: 1531 us with eight pairs per
 // row and exp and erfc evaluated for the force and for the energy, 301 us; the pipe is
 // 81% busy while a multiprocessor works.)
-__global__ void __launch_bounds__(ENVD_WARPS * 32, 4) k_env_rows_f64(DevPtrs P) {
+// The block has the tuning's size; the state of each of its warps is in dynamic shared
+// memory. (128 registers per thread at any of those sizes.)
+struct EnvdWarp {
+    float4 p[CL], shift[64];
+    double f[3 * CL][32];
+    Atom<double> i[CL];
+    int item[8];
+};
+__global__ void __launch_bounds__(ENV_WARPS_MAX * 32, 2) k_env_rows_f64(DevPtrs P) {
+    extern __shared__ __align__(16) unsigned char envd_raw[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __shared__ double s_f[ENVD_WARPS][3 * CL][32];
-    __shared__ Atom<double> s_i[ENVD_WARPS][CL];
-    __shared__ float4 s_p[ENVD_WARPS][CL];
-    __shared__ float4 s_shift[ENVD_WARPS][64];
-    __shared__ int s_item[ENVD_WARPS][8];
+    EnvdWarp& W = reinterpret_cast<EnvdWarp*>(envd_raw)[w];
     const KC<double> K = make_kc<double>(P);
     const float near2 = fmaf(P.rc2, 1e-4f, P.rc2) + 1e-5f;
     const int n_units = P.ritem_pref[P.R] * ENVD_SEG;
-    const int nw = (int)gridDim.x * ENVD_WARPS;
+    const int nw = (int)(gridDim.x * (blockDim.x >> 5));
     const unsigned int below = (1u << lane) - 1u;
-    volatile int* const I = s_item[w];
-    float4* const sh = s_shift[w];
-    double (*const fl)[32] = s_f[w];
+    volatile int* const I = W.item;
+    float4* const sh = W.shift;
+    double (*const fl)[32] = W.f;
     int unit = w * (int)gridDim.x + (int)blockIdx.x;
     while (unit < n_units) {
         __syncwarp();
@@ -573,12 +578,12 @@ __global__ void __launch_bounds__(ENVD_WARPS * 32, 4) k_env_rows_f64(DevPtrs P) 
         row_shifts(R, c, lane, sh);
         if (lane < CL) {
             const float4 x = P.xq[I[0] * CL + lane];
-            s_p[w][lane] = make_float4(x.x - c.x, x.y - c.y, x.z - c.z, 0.f);
+            W.p[lane] = make_float4(x.x - c.x, x.y - c.y, x.z - c.z, 0.f);
             Atom<double> ai = load_atom<double>(P, I[0] * CL + lane, R, K);
             ai.x -= (double)c.x;
             ai.y -= (double)c.y;
             ai.z -= (double)c.z;
-            s_i[w][lane] = ai;
+            W.i[lane] = ai;
         }
 #pragma unroll
         for (int q = 0; q < 3 * CL; ++q) fl[q][lane] = 0.0;
@@ -606,7 +611,7 @@ __global__ void __launch_bounds__(ENVD_WARPS * 32, 4) k_env_rows_f64(DevPtrs P) 
                         const float px = (x.x + u.x) - v.x, py = (x.y + u.y) - v.y, pz = (x.z + u.z) - v.z;
 #pragma unroll
                         for (int ii = 0; ii < CL; ++ii) {
-                            const float4 p = s_p[w][ii];
+                            const float4 p = W.p[ii];
                             const float dx = px - p.x, dy = py - p.y, dz = pz - p.z;
                             mask |= fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < near2 ? 1u << ii : 0u;
                         }
@@ -627,7 +632,7 @@ __global__ void __launch_bounds__(ENVD_WARPS * 32, 4) k_env_rows_f64(DevPtrs P) 
             if (mask) {
                 const int ii = __ffs(mask) - 1;
                 mask &= mask - 1u;
-                const Atom<double> ai = s_i[w][ii];
+                const Atom<double> ai = W.i[ii];
                 const double dx = a.x - ai.x, dy = a.y - ai.y, dz = a.z - ai.z;
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 if (r2 < K.rc2) {
@@ -1071,10 +1076,17 @@ __global__ void __launch_bounds__(128) k_count_lig(DevPtrs P) {
 constexpr int ENV_SMALL_ITEMS = 8;
 static bool env_small(const DevPtrs& P, int n_sm) { return P.C <= ENV_SMALL_ITEMS * n_sm; }
 
+static size_t envd_smem(int block) { return sizeof(EnvdWarp) * (size_t)(block / 32); }
+
+cudaError_t env_prepare() {
+    return cudaFuncSetAttribute(k_env_rows_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)envd_smem(ENV_WARPS_MAX * 32));
+}
+
 void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precision, int grid,
                        int block, int n_sm) {
     if (precision == 1) {
-        k_env_rows_f64<<<grid, ENVD_WARPS * 32, 0, s>>>(P);
+        k_env_rows_f64<<<grid, block, envd_smem(block), s>>>(P);
     } else if (env_small(P, n_sm)) {
         if (energy) k_env_rows<true, 1><<<grid, block, 0, s>>>(P);
         else k_env_rows<false, 1><<<grid, block, 0, s>>>(P);
@@ -1087,7 +1099,7 @@ void launch_env_forces(const DevPtrs& P, cudaStream_t s, bool energy, int precis
 int env_kernel_occupancy(int block, int precision, bool energy) {
     int nb = 0;
     if (precision == 1)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows_f64, ENVD_WARPS * 32, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows_f64, block, envd_smem(block));
     else if (energy)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_env_rows<true, 4>, block, 0);
     else
