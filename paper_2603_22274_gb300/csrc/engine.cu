@@ -374,6 +374,13 @@ StepEnd forced_end(bool rebuild, bool prune) {
 
 bool prepare_graph(abfe_ctx* c);
 
+// a build that the host forces: the ligand clusters' lists beside the environment's, as
+// in the step graph's rebuild
+void enqueue_build(abfe_ctx* c, cudaStream_t s) {
+    launch_rebuild(c->P, s, c->n_sm);
+    launch_list_build(c->P, s, c->max_lig_cl, c->fork, c->ev_fork, c->ev_join);
+}
+
 // zero forces, displacement check, rebuild and prune decisions, (predicated)
 // outer rebuild and prune
 void enqueue_prepare(abfe_ctx* c, cudaStream_t s) {
@@ -385,11 +392,14 @@ void enqueue_prepare(abfe_ctx* c, cudaStream_t s) {
     launch_integrate(with_sp(c, SP_ZERO), s, c->n_sm, forced_end(c->force_rebuild, c->force_prune));
     // host-forced builds and prunes are timed while profiling is on
     const bool tb = c->force_rebuild, tp = c->force_rebuild || c->force_prune;
-    if (tb) prof_rec(c, c->ev_build, true, s);
-    launch_rebuild(c->P, s, c->n_sm);
-    if (tb) launch_list_build(c->P, s, c->max_lig_cl, c->fork, c->ev_fork, c->ev_join);
-    else launch_list_build(c->P, s, c->max_lig_cl);
-    if (tb) prof_rec(c, c->ev_build, false, s);
+    if (tb) {
+        prof_rec(c, c->ev_build, true, s);
+        enqueue_build(c, s);
+        prof_rec(c, c->ev_build, false, s);
+    } else {
+        launch_rebuild(c->P, s, c->n_sm);
+        launch_list_build(c->P, s, c->max_lig_cl);
+    }
     if (tp) prof_rec(c, c->ev_prune, true, s);
     launch_prune(c->P, s, c->n_sm);
     if (tp) prof_rec(c, c->ev_prune, false, s);
@@ -2555,8 +2565,7 @@ abfe_status abfe_autotune_cadence(abfe_ctx* c, double dt, double gamma, uint64_t
     auto timed = [&](bool rebuild, float& build_ms, float& prune_ms, float& env_ms) -> bool {
         launch_integrate(with_sp(c, SP_ZERO), c->stream, c->n_sm, forced_end(rebuild, true));
         cudaEventRecord(e0, c->stream);
-        launch_rebuild(c->P, c->stream, c->n_sm);
-        launch_list_build(c->P, c->stream, c->max_lig_cl);
+        enqueue_build(c, c->stream);
         cudaEventRecord(e1, c->stream);
         launch_prune(c->P, c->stream, c->n_sm);
         cudaEventRecord(e2, c->stream);
