@@ -219,7 +219,7 @@ void abfe_set_allocator(abfe_alloc_fn alloc_fn, abfe_free_fn free_fn, void *user
 /* Create a context for n_replicas windows. systems[0..n_systems) are the
  * distinct structures; replica r simulates systems[system_of_replica[r]]
  * (replicas of one system start from identical coordinates). cuda_stream is a
- * cudaStream_t (NULL = legacy default stream). Fails with
+ * cudaStream_t (NULL: the context creates a stream of its own). Fails with
  * ABFE_ERR_CUTOFF_TOO_LARGE if r_c >= L/2, ABFE_ERR_INVALID_ARG for bad
  * indices, parameters or sizes. */
 abfe_status abfe_create(const abfe_system_desc *systems, int32_t n_systems,
@@ -248,7 +248,8 @@ abfe_status abfe_compute(abfe_ctx *ctx, double *h_forces, double *h_energy, doub
 
 /* Same evaluation with device outputs: d_forces [total_atoms][3] float
  * (original order) or NULL, d_energy [R][ABFE_N_ENERGY] double or NULL,
- * d_dudl [R][ABFE_N_DUDL] double or NULL. Stream-ordered, no host sync. */
+ * d_dudl [R][ABFE_N_DUDL] double or NULL. Stream-ordered, no host sync; inside a
+ * capture of the stream it launches directly. */
 abfe_status abfe_compute_device(abfe_ctx *ctx, float *d_forces, double *d_energy, double *d_dudl);
 
 /* Advance every replica by n_steps BAOAB Langevin steps (B A O A, forces, B)

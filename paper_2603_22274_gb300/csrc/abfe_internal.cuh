@@ -52,7 +52,11 @@ constexpr int ERFC_NT = 1025, ERFC_INV_H = 128;
 // FP64 pair kernels: warps per item of the row kernel, idle lanes that make it refill,
 // warps per item of the ligand kernel (12 frames of 672 atoms: row kernel's 1, 2, 4, 8
 // per item 501, 476, 550, 608 us a pass; refills at 4, 8, 12 idle lanes 502, 502, 511;
-// ligand kernel's 1, 2, 4 per item 476, 458, 457)
+// ligand kernel's 1, 2, 4 per item 476, 458, 457). Larger systems: the row kernel's 1,
+// 2, 4 per item take 354, 343, 324 us a pass for one window of 4,500 atoms, 865, 887,
+// 993 for four and 1050, 1106, 1265 for one of 25,000 (with many items, one warp each
+// idles fewer lanes); refills and the ligand kernel's 4 change these by 2% at most, its
+// 1 the first by 5%.
 constexpr int ENVD_SEG = 2, ENVD_REFILL = 8, LIGD_SEG = 2;
 constexpr int COL_MAX = 1024;       // atoms per column (per-column sort capacity)
 constexpr double FSCALE = 4294967296.0;
@@ -61,7 +65,9 @@ constexpr double INV_FSCALE = 1.0 / 4294967296.0;
 constexpr float DUMMY_FAR = 1.0e4f;
 // j-cluster entries per ligand work item (a warp each). Shorter than the
 // environment's: one window's ligand has some 2,300 entries in all, and in items
-// of 16 they kept 144 of the chip's 608 schedulers busy for 25 us.
+// of 16 they kept 144 of the chip's 608 schedulers busy for 25 us. The item regions,
+// sized for every cluster under every image, are twice those for 16 (1,152 windows:
+// 0.4 GB).
 constexpr int LIG_CHUNK = 8;
 
 // error bits (Counters::err)

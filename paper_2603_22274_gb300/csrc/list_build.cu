@@ -757,7 +757,8 @@ __device__ void build_group(const DevPtrs& P, LBS<ECAP, HCAP, XCAP, GM>& L, int 
         // images kz with z_j + kz Lz in [zlo, zhi] for some z_j in [0, Lz) (most groups:
         // one). With one image the order of the segments is that of the columns, so
         // columns out of reach or on the wrong side of the half-list rule are
-        // dropped before the batches of 32 are formed.
+        // dropped before the batches of 32 are formed. (A column fits the key's 26 bits:
+        // each has a cluster of eight slots set aside, and slots are numbered in 27 bits.)
         int n_kz = 0;
         for (int kz = -1; kz <= 1; ++kz) n_kz += zhi - kz * Lz >= 0.f && zlo - kz * Lz < Lz ? 1 : 0;
         const int n_wrap = is_lig ? -1 : n_env;
@@ -769,7 +770,7 @@ __device__ void build_group(const DevPtrs& P, LBS<ECAP, HCAP, XCAP, GM>& L, int 
             if (lane == 0) L.n_col = 0;
             __syncwarp();
             {
-                int key = -1;   // column | kx + 1 << 28 | ky + 1 << 30
+                int key = -1;   // column | kx + 1 << 26 | ky + 1 << 28
                 while (cb < ncand && (n_kz > 1 ? n_q == 0 : n_q < 32)) {
                     const int q = cb + lane;
                     cb += 32;

@@ -395,9 +395,9 @@ __device__ __forceinline__ void env_tail_row(const DevPtrs& P, const volatile in
 //
 // The item and the claim counters live in shared memory (volatile: read again
 // where they are needed), so that 64 registers hold the round loop: with them in
-// registers it spilled inside the loop, which cost more than the atom of the
-// next round loaded ahead gained (24 x 25k atoms: 429 us with the prefetch, 472
-// with this claim scheme in registers too, 427 as it is).
+// registers it spilled inside the loop (24 x 25k atoms: 472 us, 427 from shared
+// memory). On that workload it buys the claim scheme and no time: the prefetch of
+// the next round's atom with the former claims, in registers, took 429.
 template <bool ENERGY, int MINB>
 __global__ void __launch_bounds__(256, MINB) k_env_rows(DevPtrs P) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1072,7 +1072,16 @@ __global__ void __launch_bounds__(128) k_count_lig(DevPtrs P) {
 // Small systems: at most ENV_SMALL_ITEMS clusters per SM give each scheduler a
 // warp or two, whatever the registers allow: there the kernel is bound by one
 // warp's latency, and the variant with 255 registers interleaves the eight pairs
-// of a row.
+// of a row. Both variants add the same bits. Windows of 4,500 atoms (4.2 clusters per
+// SM each), us of a step in the graph and of a whole energy pass with 64 | 255
+// registers, for 256-thread blocks (items of up to 512 entries) and 128 (up to 64):
+//   clusters per SM     4.2         8.3         17          33         66        265
+//   step, 256       48.5|46.8   65.0|53.0   71.0|68.7   81.7|85.5   133|141   408|458
+//   step, 128       52.4|54.0   58.0|61.5   70.3|74.5   93.5|101    142|155   465|522
+//   energy, 256     84.5|80.0    121|89.0    124|105     130|125    206|196   574|592
+//   energy, 128     77.2|78.1   97.3|85.4    112|101     144|131    210|192   666|610
+// Steps with 256-thread blocks gain up to 17 clusters per SM, with 128 they lose 3 to
+// 6%; energy passes gain at both, and on beyond the line.
 constexpr int ENV_SMALL_ITEMS = 8;
 static bool env_small(const DevPtrs& P, int n_sm) { return P.C <= ENV_SMALL_ITEMS * n_sm; }
 

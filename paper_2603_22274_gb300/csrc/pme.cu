@@ -200,8 +200,6 @@ __device__ __forceinline__ C cmul(C a, C b) {
     return cx<C>::mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// one Stockham stage of radix RAD on a line of n points (warp-cooperative)
-// tw[k] = exp(-2 pi i k / n), k < n, in shared memory
 // small integers: q = floor(j / d) from a float reciprocal (exact for j < 2^20)
 __device__ __forceinline__ int fdiv(int j, float inv_d) { return (int)(((float)j + 0.5f) * inv_d); }
 
@@ -251,7 +249,8 @@ __device__ __forceinline__ void butterfly(const C (&v)[RAD], C (&y)[RAD]) {
     }
 }
 
-// One radix-RAD Stockham stage of a line whose points lie st elements apart.
+// One radix-RAD Stockham stage, by a warp, of a line whose n points lie st elements
+// apart; tw[k] = exp(-2 pi i k / n), k < n, in shared memory.
 template <int RAD, class C>
 __device__ __forceinline__ void fft_stage(const C* src, C* dst, int st, const C* tw, int n, int Ns, int lane) {
     const int m = n / RAD;
