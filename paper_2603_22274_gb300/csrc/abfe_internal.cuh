@@ -493,7 +493,7 @@ void launch_bonds(const DevPtrs& P, cudaStream_t s, int precision, bool energy);
 // alchemical waters: slot charges at every replica's lambda_q; energy-pass sums
 void launch_aw_refresh(const DevPtrs& P, cudaStream_t s);
 void launch_aw_sums(const DevPtrs& P, cudaStream_t s, int max_aw, int max_cl);
-void launch_restraints(const DevPtrs& P, cudaStream_t s);
+void launch_restraints(const DevPtrs& P, cudaStream_t s, int max_tors);
 void launch_finalize(const DevPtrs& P, cudaStream_t s);
 void launch_ukn_assemble(const DevPtrs& P, cudaStream_t s, double kT);
 void launch_scatter_out(const DevPtrs& P, cudaStream_t s, int what, double* outd, float* outf,

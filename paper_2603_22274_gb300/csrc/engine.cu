@@ -75,7 +75,7 @@ struct abfe_ctx {
     std::vector<int64_t> rep_atom_off;
     int64_t total_atoms = 0;
     int S = 0, C = 0, NCOL = 0, max_bonds = 0, n_lig_cl = 0, max_lig_cl = 0, max_cl_cap = 0;
-    int n_bond_total = 0;
+    int n_bond_total = 0, max_tors = 0;
     int64_t epc_max = 0;                   // outer entries per cluster, the largest estimate
     int max_aw = 0;
     std::vector<int> sys_tors_off, sys_ntors, sys_aw_off, sys_naw;
@@ -338,7 +338,7 @@ void enqueue_forces(abfe_ctx* c, cudaStream_t s, bool energy, bool fork = true) 
     launch_lig_forces(c->P, f, c->prm.precision, c->lig_grid, 128, energy);
     if (fork) prof_rec(c, c->ev_lig, false, f);
     launch_bonds(c->P, f, c->prm.precision, energy);
-    launch_restraints(c->P, c->pme ? f : f2);
+    launch_restraints(c->P, c->pme ? f : f2, c->max_tors);
     if (energy) launch_aw_sums(c->P, f2, c->max_aw, c->max_cl_cap);
     if (c->pme) {
         launch_pme_forces(c->P, c->pm, f2, c->n_sm, energy, energy ? c->ev_pme : nullptr);
@@ -974,6 +974,7 @@ abfe_status abfe_create(const abfe_system_desc* systems, int32_t n_systems,
         }
         c->sys_tors_off.push_back((int)h_tors.size());
         c->sys_ntors.push_back(d.n_torsions);
+        c->max_tors = std::max(c->max_tors, d.n_torsions);
         for (int k = 0; k < d.n_torsions; ++k) {
             const int32_t* q = d.torsion_idx + 4 * k;
             h_tors.push_back(make_int4(q[0], q[1], q[2], q[3]));

@@ -7,7 +7,7 @@
 //   last prune; its last block ends the step (step counter, rebuild and prune
 //   flags, CUDA-graph conditionals).
 // * k_bonds: harmonic bonds (keep the synthetic molecules together).
-// * k_restraints: the FP64 bonded terms, a block per replica: the six-term Boresch
+// * k_restraints: the FP64 bonded terms, blocks per replica: the six-term Boresch
 //   restraint (paper, section "Restraints") and the periodic torsions of the
 //   ligand's rotatable bonds, scaled by lambda_v when annihilating (paper,
 //   section "Double annihilation protocol").
@@ -572,22 +572,27 @@ __device__ double torsion_term(const DevPtrs& P, const RepDev& R, int t) {
     return prm.x * (1.0 + (cn * prm.z + sn * prm.w));
 }
 
-// The FP64 bonded terms of a replica (block): warps 0-2 take its torsions, warp 3
-// the angles and the dihedrals of its Boresch restraint, warp 2 the restraint's
-// distance. Bound by FP64 latency (63 issue cycles per warp instruction on this
+// The FP64 bonded terms of a replica: warps 0-2 of its blocks take TORS_BLOCK torsions
+// each, warp 3 of its first block the angles and the dihedrals of its Boresch restraint,
+// warp 2 the restraint's distance. Bound by FP64 latency (63 issue cycles per warp instruction on this
 // chip), so the restraint's terms run on lanes of their own and no term calls a
 // trigonometric function but acos: 54 us (restraint, one thread per replica) and
 // 17 us (torsions, atan2 + cos + sin) in two launches before, 18 us together now,
-// 12 with torsions alone.
+// 12 with torsions alone. A round of 96 torsions takes 6 us, so more of them take more
+// blocks: a step of one window of 4,500 atoms with 11, 176, 352, 704, 1,408 torsions took
+// 54, 57, 69, 98, 155 us in one block per window, 54, 55, 56, 55, 56 so.
+constexpr int TORS_BLOCK = 96;
 __global__ void __launch_bounds__(128) k_restraints(DevPtrs P) {
-    const int rep = blockIdx.x;
+    const int rep = blockIdx.x, seg = blockIdx.y;
     const RepDev& R = P.reps[rep];
+    if (seg > 0 && seg * TORS_BLOCK >= R.n_tors) return;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __shared__ double s_b[6], s_t[3];
     double et = 0.0;
     if (w < 3)
-        for (int t = threadIdx.x; t < R.n_tors; t += 96) et += torsion_term(P, R, t);
-    if (R.boresch >= 0) {
+        for (int t = seg * TORS_BLOCK + threadIdx.x; t < R.n_tors; t += (int)gridDim.y * TORS_BLOCK)
+            et += torsion_term(P, R, t);
+    if (seg == 0 && R.boresch >= 0) {
         const BoreschDev& B = P.bor[R.boresch];
         if (w == 3 && lane < 5) s_b[lane + 1] = boresch_term(P, R, B, lane + 1);
         if (w == 2 && lane == 31) s_b[0] = boresch_term(P, R, B, 0);
@@ -597,8 +602,8 @@ __global__ void __launch_bounds__(128) k_restraints(DevPtrs P) {
     if (w < 3 && lane == 0) s_t[w] = et;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const double U = R.boresch < 0 ? 0.0 : s_b[0] + s_b[1] + s_b[2] + s_b[3] + s_b[4] + s_b[5];
-        P.eb[rep] = U;
+        const double U = seg > 0 || R.boresch < 0 ? 0.0 : s_b[0] + s_b[1] + s_b[2] + s_b[3] + s_b[4] + s_b[5];
+        if (seg == 0) P.eb[rep] = U;
         const double tt = s_t[0] + s_t[1] + s_t[2];
         if (!isfinite(tt) || !isfinite(U)) set_err(P.cnt, ERRB_NONFINITE, rep);
         if (tt != 0.0) {
@@ -888,8 +893,9 @@ void launch_aw_sums(const DevPtrs& P, cudaStream_t s, int max_aw, int max_cl) {
     k_aw_sums<<<dim3(max_aw, P.R, min((max_cl * CL + AW_SEG - 1) / AW_SEG, 4096)), 128, 0, s>>>(P);
 }
 
-void launch_restraints(const DevPtrs& P, cudaStream_t s) {
-    k_restraints<<<P.R, 128, 0, s>>>(P);
+void launch_restraints(const DevPtrs& P, cudaStream_t s, int max_tors) {
+    const int segs = max(1, min((max_tors + TORS_BLOCK - 1) / TORS_BLOCK, 65535));
+    k_restraints<<<dim3(P.R, segs), 128, 0, s>>>(P);
 }
 
 void launch_finalize(const DevPtrs& P, cudaStream_t s) {
